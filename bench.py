@@ -39,6 +39,8 @@ PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 PROFILE_FILE = os.path.join(ROOT, "profiles", "rd_step_brusselator_256.md")
 WORKLOAD = "brusselator_256^3_periodic_10000_steps"
 KERNEL_SOURCES = ["paper_1004_0480_gb300/csrc/rd_step_kernel.cuh",
+                  "paper_1004_0480_gb300/csrc/rd_march_kernel.cuh",
+                  "paper_1004_0480_gb300/csrc/rd_pack.cuh",
                   "paper_1004_0480_gb300/csrc/rd_step1w_kernel.cuh",
                   "paper_1004_0480_gb300/csrc/rd_debug.cuh",
                   "paper_1004_0480_gb300/csrc/rd_k_brusselator.cu",
@@ -354,7 +356,7 @@ def run_ours(args, ws, rank, local):
                 "frac": achieved / peak,
                 "traffic": traffic, "traffic_tuning": traffic_tun,
                 "peak_source": peak_src,
-                "kernel": ("rd_step1_kernel<MBrusselator,float>" if T == 1
+                "kernel": (f"rd_march_kernel<MBrusselator,float,{T}>" if T <= 2
                            else f"rd_step_kernel<MBrusselator,float,{T}>"),
                 "algorithmic_bytes_per_launch": bytes_per_launch,
                 "launch_ms": per_launch_ms,

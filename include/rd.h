@@ -288,12 +288,14 @@ rd_status rd_set_step_count(rd_ctx* ctx, int64_t n);
  * rd_set_tuning validates; RD_EINVAL if the CTA or its shared memory does
  * not fit one SM.  A new context starts with tsteps 1, tile_y 14 (12 for
  * the Cahn-Hilliard models), graph 1, regcap 0 and the z-chunk whose work
- * items fill the resident CTA slots in the fewest waves. */
+ * items fill the resident CTA slots in the fewest waves.  Until a tuning is
+ * set (rd_set_tuning, rd_autotune) the library may step with another tiling
+ * and with two steps per launch where its cost model expects that to be
+ * faster: the results are the same bits, rd_launch_count is lower. */
 typedef struct rd_tuning {
     int32_t tsteps, tile_q, tile_y, zchunk, graph;
-    int32_t regcap;   /* 1: cap the 7-point one-step kernel at 64 registers
-                         per thread (more resident warps), 0: let it use up
-                         to 128; the 19-point kernel ignores it              */
+    int32_t regcap;   /* 0 or 1; no effect: each kernel has its own register
+                         budget                                              */
 } rd_tuning;
 rd_status rd_get_tuning(const rd_ctx* ctx, rd_tuning* out);
 rd_status rd_set_tuning(rd_ctx* ctx, const rd_tuning* t);

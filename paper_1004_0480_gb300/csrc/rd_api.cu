@@ -252,6 +252,10 @@ struct rd_ctx {
     bool own_stream = false;
     cudaStream_t capture_stream = nullptr;
     rd_tuning tun{};
+    // what the library itself steps with while the tuning is the default one
+    // (plan.tsteps 0: the tuning as it is), with the descriptors
+    rd_tuning plan{}, plan1{};     // plan1: for calls of one step
+    InstDesc plan_desc{}, plan1_desc{};
     int kernel = RD_KERNEL_MARCH;  // step kernel (rd_set_kernel)
     bool desc_dirty = true;
     InstDesc desc{};
@@ -559,6 +563,78 @@ rd_tuning default_tuning(const rd_config& g) {
     return t;
 }
 
+// Cost of a plane of one work item, in microseconds: a + b x (tile rows
+// resident on the SM), fitted to sweeps of tile heights and z-chunks on a
+// GB300 (grids of 32^3 to 512^3, see rd_march_kernel.cuh for the rates).  An
+// SM marches the rows of its CTAs at one rate, so more CTAs or taller tiles
+// cost the same per row; what a small grid saves is planes per item.
+struct PlaneCost {
+    double a, b;
+};
+PlaneCost plane_cost(int nspecies, int storage, int T) {
+    const bool h = storage == RD_STORE_BF16;
+    switch (nspecies) {
+    case 1: return T == 2 ? PlaneCost{0.20, 0.0135} : PlaneCost{0.17, 0.0085};
+    case 2:
+        if (h) return T == 2 ? PlaneCost{0.30, 0.0197} : PlaneCost{0.30, 0.0079};
+        return T == 2 ? PlaneCost{0.10, 0.0335} : PlaneCost{0.15, 0.0185};
+    default: return T == 2 ? PlaneCost{0.40, 0.0770} : PlaneCost{0.30, 0.0340};
+    }
+}
+// launch gap and pipeline fill of a launch (replayed from a graph)
+constexpr double kLaunchUs = 2.4;
+
+// What a context steps with while its tuning is the default one: the tile
+// height, z-chunk and steps per launch (at most ``maxT``) of the least
+// modelled cost per step.  Small grids take short chunks (a 97 x 65 x 50
+// Brusselator: 12 rows x 2 planes, 3.0 us a step, where 14 rows x 8 planes
+// at one step per launch took 9.8), large ones the fewest waves; two steps
+// per launch halve the launches and the traffic, but three-species and
+// bfloat16 problems are bound by their arithmetic and keep one where the
+// launch gap does not decide.
+rd_tuning default_plan(const rd_config& g, const rd_tuning& t1, int maxT) {
+    rd_tuning best = t1;
+    if (is_ch(g.model) || stencil_of(g) == 19) {   // no plan: the tuning as it is
+        best.tsteps = 0;
+        return best;
+    }
+    const int sms = num_sms();
+    double best_cost = -1.0;
+    for (int T = 1; T <= std::min(maxT, max_tsteps(g)); ++T)
+        for (int ty = 16; ty >= 6; ty -= 2) {
+            rd_tuning t = t1;
+            t.tsteps = T;
+            t.tile_y = ty;
+            t.zchunk = 1;
+            if (T > 2 || check_tuning(g, t) != RD_OK) continue;
+            const int occ = occupancy(g.model, g.storage, T, ty, 0, variant_code(g), 7);
+            if (occ < 1) continue;
+            const PlaneCost pc = plane_cost(g.nspecies, g.storage, T);
+            const long long cols = (long long)tiles(g.nx, kTileW) * tiles(g.ny, ty);
+            const long long slots = (long long)occ * sms;
+            int last = 0;
+            for (int k = 1; k <= g.nz; ++k) {
+                const int zc = tiles(g.nz, k);
+                if (zc == last) continue;
+                last = zc;
+                const long long items = cols * tiles(g.nz, zc);
+                const long long full = items / slots, rest = items % slots;
+                const long long rows = tiles((int)rest, sms) * (long long)ty;
+                const double planes = zc + 2 * (T - 1) + 1;
+                const double us =
+                    planes * (full * (pc.a + pc.b * occ * ty) + (rest ? pc.a + pc.b * rows : 0.0));
+                const double cost = (kLaunchUs + us) / T;
+                if (best_cost < 0 || cost < best_cost) {
+                    best_cost = cost;
+                    best = t;
+                    best.zchunk = zc;
+                }
+                if (us > 64 * kLaunchUs && zc < 16) break;   // large grid: no shorter chunks
+            }
+        }
+    return best;
+}
+
 void fill_desc(rd_ctx* c, InstDesc& d, const rd_tuning& t) {
     const rd_config& g = c->cfg;
     std::memset(&d, 0, sizeof(d));
@@ -658,6 +734,10 @@ bool plain_problem(const rd_config& g) {
 rd_status upload_desc(rd_ctx* c) {
     if (!c->desc_dirty) return RD_OK;
     fill_desc(c, c->desc, c->tun);
+    if (c->plan.tsteps) {
+        fill_desc(c, c->plan_desc, c->plan);
+        fill_desc(c, c->plan1_desc, c->plan1);
+    }
     RD_CUDA(c, cudaMemcpyAsync(c->desc_dev, &c->desc, sizeof(InstDesc), cudaMemcpyHostToDevice,
                                c->stream));
     RD_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -692,20 +772,27 @@ rd_status finish_setup(rd_ctx* c) {
     return upload_desc(c);
 }
 
+// Which tuning a launch takes: the context's, or the library's plans.
+enum class Use { kTuning, kPlan, kPlan1 };
+const rd_tuning& tuning_of(const rd_ctx* c, Use u) {
+    return u == Use::kPlan ? c->plan : u == Use::kPlan1 ? c->plan1 : c->tun;
+}
+
 // One fused launch advancing T steps, reading level ``c->cur``.
-rd_status launch_ctx(rd_ctx* c, int T, int parity, cudaStream_t st) {
+rd_status launch_ctx(rd_ctx* c, int T, int parity, cudaStream_t st, Use use = Use::kTuning) {
+    const rd_tuning& t = tuning_of(c, use);
     LaunchArgs a{};
     a.desc = c->desc_dev;
     a.ninst = 1;
     a.parity = parity;
-    a.nitems = items_of(c->desc);
     a.use_one = 1;
-    a.one = c->desc;
-    a.regcap = c->tun.regcap;
+    a.one = use == Use::kPlan ? c->plan_desc : use == Use::kPlan1 ? c->plan1_desc : c->desc;
+    a.nitems = items_of(a.one);
+    a.regcap = t.regcap;
     a.plain = plain_problem(c->cfg);
     a.wind3 = c->cfg.wind_kind == RD_WIND_3D;
-    a.vw = vw_of(c->tun.tile_q);
-    a.ty = c->tun.tile_y;
+    a.vw = vw_of(t.tile_q);
+    a.ty = t.tile_y;
     if (c->kernel == RD_KERNEL_RESIDENT) {
         // T steps in one cooperative launch (zeroed barrier count and word)
         RD_CUDA(c, cudaMemsetAsync(c->bar, 0, 2 * sizeof(unsigned), st));
@@ -726,10 +813,10 @@ rd_status launch_ctx(rd_ctx* c, int T, int parity, cudaStream_t st) {
         return RD_OK;
     }
     const int sten = stencil_of(c->cfg);
-    const size_t sm = smem_of(c->cfg.model, c->cfg.storage, T, a.ty, sten, c->tun.tile_q);
+    const size_t sm = smem_of(c->cfg.model, c->cfg.storage, T, a.ty, sten, t.tile_q);
     const int occ = std::max(
         1, occupancy(c->cfg.model, c->cfg.storage, T, a.ty, a.regcap,
-                     a.plain ? 1 : a.wind3 ? 2 : 0, sten, c->tun.tile_q));
+                     a.plain ? 1 : a.wind3 ? 2 : 0, sten, t.tile_q));
     const long long grid = std::min<long long>(a.nitems, (long long)occ * num_sms());
     cudaError_t e =
         launch_model(c->cfg.model, c->cfg.storage, T, a, (int)grid, sm, st, nullptr, sten);
@@ -738,16 +825,16 @@ rd_status launch_ctx(rd_ctx* c, int T, int parity, cudaStream_t st) {
     return RD_OK;
 }
 
-long long ctx_graph_key(const rd_ctx* c) {
-    const rd_tuning& t = c->tun;
+long long ctx_graph_key(const rd_ctx* c, const rd_tuning& t) {
     return ((((((long long)t.tsteps * 64 + t.tile_q) * 64 + t.tile_y) * 100000 + t.zchunk) * 2 +
              t.regcap) * 4 + c->kernel);
 }
 
 constexpr int kGraphLaunches = 16;
 
-rd_status build_ctx_graph(rd_ctx* c) {
-    const long long key = ctx_graph_key(c);
+rd_status build_ctx_graph(rd_ctx* c, Use use) {
+    const rd_tuning& t = tuning_of(c, use);
+    const long long key = ctx_graph_key(c, t);
     if (c->graph.exec && c->graph.key == key) return RD_OK;
     c->graph.reset();
     if (!c->capture_stream)
@@ -756,7 +843,7 @@ rd_status build_ctx_graph(rd_ctx* c) {
     const int64_t before = c->launches;
     rd_status st = RD_OK;
     for (int i = 0; i < kGraphLaunches && st == RD_OK; ++i)
-        st = launch_ctx(c, c->tun.tsteps, i & 1, c->capture_stream);
+        st = launch_ctx(c, t.tsteps, i & 1, c->capture_stream, use);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(c->capture_stream, &g);
     if (st != RD_OK) { if (g) cudaGraphDestroy(g); return st; }
@@ -766,7 +853,7 @@ rd_status build_ctx_graph(rd_ctx* c) {
     if (e != cudaSuccess) return cuda_fail(c, e, "graph instantiate");
     c->graph.launches = (int)(c->launches - before);   // kernels in the graph
     c->launches = before;                               // captured, not run
-    c->graph.tsteps = c->tun.tsteps;
+    c->graph.tsteps = t.tsteps;
     c->graph.key = key;
     return RD_OK;
 }
@@ -799,14 +886,18 @@ rd_status step_ctx(rd_ctx* c, int64_t n) {
         c->steps += n;
         return RD_OK;
     }
-    const int T = c->tun.tsteps;
+    const Use use = c->plan.tsteps == 0 || c->kernel != RD_KERNEL_MARCH ? Use::kTuning
+                    : n >= c->plan.tsteps                               ? Use::kPlan
+                                                                        : Use::kPlan1;
+    const rd_tuning& t = tuning_of(c, use);
+    const int T = t.tsteps;
     int64_t full = n / T;
     const int rem = (int)(n % T);
-    if (c->tun.graph && full >= kGraphLaunches) {
-        st = build_ctx_graph(c);
+    if (t.graph && full >= kGraphLaunches) {
+        st = build_ctx_graph(c, use);
         if (st != RD_OK) return st;
         if (c->cur == 1) {   // the graph starts from level 0
-            if ((st = launch_ctx(c, T, 1, c->stream)) != RD_OK) return st;
+            if ((st = launch_ctx(c, T, 1, c->stream, use)) != RD_OK) return st;
             c->cur = 0;
             --full;
         }
@@ -818,11 +909,11 @@ rd_status step_ctx(rd_ctx* c, int64_t n) {
         }
     }
     for (int64_t i = 0; i < full; ++i) {
-        if ((st = launch_ctx(c, T, c->cur, c->stream)) != RD_OK) return st;
+        if ((st = launch_ctx(c, T, c->cur, c->stream, use)) != RD_OK) return st;
         c->cur ^= 1;
     }
     if (rem) {
-        if ((st = launch_ctx(c, rem, c->cur, c->stream)) != RD_OK) return st;
+        if ((st = launch_ctx(c, rem, c->cur, c->stream, use)) != RD_OK) return st;
         c->cur ^= 1;
     }
     c->steps += n;
@@ -925,6 +1016,8 @@ rd_status rd_create(const rd_config* cfg, rd_ctx** out) {
     if (e != cudaSuccess) { delete c; return cuda_fail(nullptr, e, "cudaStreamCreate"); }
     c->own_stream = true;
     c->tun = default_tuning(c->cfg);
+    c->plan = default_plan(c->cfg, c->tun, 2);
+    c->plan1 = default_plan(c->cfg, c->tun, 1);
     if (!(cfg->flags & RD_FLAG_NO_ALLOC)) {
         // owned from the first allocation on, so rd_destroy frees whatever
         // was obtained when a later one fails
@@ -1182,6 +1275,7 @@ rd_status rd_set_tuning(rd_ctx* c, const rd_tuning* t) {
     if (st != RD_OK) return fail(c, st, "%s", g_err);
     c->tun = *t;
     c->tun.zchunk = std::min(c->tun.zchunk, c->cfg.nz);
+    c->plan.tsteps = 0;
     c->desc_dirty = true;
     return RD_OK;
 }
@@ -1199,6 +1293,7 @@ rd_status rd_autotune(rd_ctx* c, rd_tuning* best_out) {
         auto it = g_tune_cache.find(key);
         if (it != g_tune_cache.end() && check_tuning(g, it->second) == RD_OK) {
             c->tun = it->second;
+            c->plan.tsteps = 0;
             c->desc_dirty = true;
             if (best_out) *best_out = c->tun;
             return RD_OK;
@@ -1216,31 +1311,26 @@ rd_status rd_autotune(rd_ctx* c, rd_tuning* best_out) {
         // 8 cells per thread: the one-step 7-point kernel (heights 4k)
         if (tq == 8 && (T != 1 || is_ch(g.model) || sten != 7)) continue;
         for (int ty : {4, 8, 10, 12, 14, 16, 20, 24, 28, 32}) {
-          // the register cap is a variant of the 7-point 4-cell one-step kernel
-          const bool rc_variant = T == 1 && !is_ch(g.model) && sten == 7 && tq == kTileQ;
-          for (int rc = 0; rc <= (rc_variant ? 1 : 0); ++rc) {
             rd_tuning t{};
             t.tsteps = T; t.tile_q = tq; t.tile_y = ty; t.graph = 1; t.zchunk = 1;
-            t.regcap = rc;
             if (check_tuning(g, t) != RD_OK) continue;
-            const int occ = occupancy(g.model, g.storage, T, ty, rc, variant_code(g), sten, tq);
+            const int occ = occupancy(g.model, g.storage, T, ty, 0, variant_code(g), sten, tq);
             if (occ < 1) continue;
-            // z-chunks for 1, 2, 4, 8 waves of CTAs; for one step per launch
-            // also every split of z into 1..16 chunks, since how evenly the
-            // items fill the CTA slots decides as much as the tile does
+            // z-chunks for 1, 2, 4, 8 waves of CTAs; for the one- and two-step
+            // kernels also every split of z into 1..16 chunks, since how
+            // evenly the items fill the CTA slots decides as much as the tile
             std::vector<int> zcs;
             for (int waves : {1, 2, 4, 8}) zcs.push_back(auto_zchunk(g, t, occ, waves));
-            if (T == 1)
+            if (T == 1 || (T == 2 && !is_ch(g.model) && !(ty & 1)))
                 for (int k = 1; k <= 16; ++k) zcs.push_back((g.nz + k - 1) / k);
             for (int zc : zcs) {
                 t.zchunk = zc;
                 bool dup = false;
                 for (auto& o : cands)
                     dup |= (o.tsteps == t.tsteps && o.tile_q == t.tile_q && o.tile_y == t.tile_y &&
-                            o.zchunk == t.zchunk && o.regcap == t.regcap);
+                            o.zchunk == t.zchunk);
                 if (!dup) cands.push_back(t);
             }
-          }
         }
       }
     cudaEvent_t e0, e1;
@@ -1300,6 +1390,7 @@ rd_status rd_autotune(rd_ctx* c, rd_tuning* best_out) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     c->tun = best > 0 ? bt : saved;
+    if (best > 0) c->plan.tsteps = 0;
     c->desc_dirty = true;
     if (best > 0) {
         std::lock_guard<std::mutex> lk(g_tune_mu);

@@ -5,6 +5,9 @@
 #pragma once
 
 #include "rd_internal.h"
+#ifdef __CUDACC__
+#include "rd_pack.cuh"
+#endif
 
 namespace rdk {
 
@@ -13,13 +16,15 @@ namespace rdk {
 struct MTuring {
     static constexpr int S = 2;
     static constexpr bool CH = false;
-    __device__ __forceinline__ static void react(const InstDesc& d, const float* c, float* inc) {
-        const float c1 = c[0], c2 = c[1];
-        const float cube = __fmul_rn(__fmul_rn(c1, c1), c1);
-        const float f = __fsub_rn(__fsub_rn(c1, cube), c2);
-        const float g = __fmul_rn(d.p[2], __fsub_rn(__fmaf_rn(-d.p[0], c2, c1), d.p[1]));
-        inc[0] = __fmul_rn(d.dt, f);
-        inc[1] = __fmul_rn(d.dt, g);
+    template <class V>
+    __device__ __forceinline__ static void react(const InstDesc& d, const V* c, V* inc) {
+        const V c1 = c[0], c2 = c[1];
+        const V cube = vmul_rounded(vmul(c1, c1), c1);
+        const V f = vsub(vsub(c1, cube), c2);
+        const V g = vmul(vset<V>(d.p[2]),
+                         vadd(vfma(vset<V>(-d.p[0]), c2, c1), vset<V>(-d.p[1])));
+        inc[0] = vmul(vset<V>(d.dt), f);
+        inc[1] = vmul(vset<V>(d.dt), g);
     }
 };
 #endif

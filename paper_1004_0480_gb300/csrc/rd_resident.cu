@@ -333,15 +333,7 @@ rd_resident_kernel(const __grid_constant__ LaunchArgs a, const ResidentPlan p, i
                     float cen[S][kVEC], inc[S][kVEC];
 #pragma unroll
                     for (int s = 0; s < S; ++s) Store<ST>::load(src + s * fsm + own + xs, cen[s]);
-#pragma unroll
-                    for (int e = 0; e < kVEC; ++e) {
-                        float cv[S], iv[S];
-#pragma unroll
-                        for (int s = 0; s < S; ++s) cv[s] = cen[s][e];
-                        M::react(sd, cv, iv);
-#pragma unroll
-                        for (int s = 0; s < S; ++s) inc[s][e] = iv[s];
-                    }
+                    react4<M>(sd, cen, inc);
                     const float cx = PLAIN ? 0.0f : courant_at(sd, sd.courant, z);
                     const bool src_here = sd.src_s >= 0 && y == sd.src_y && z == sd.src_z;
                     const unsigned faces = xy_faces(xs, y, nx, ny) | z_faces(z, nz);
@@ -363,10 +355,7 @@ rd_resident_kernel(const __grid_constant__ LaunchArgs a, const ResidentPlan p, i
                         }
                         if constexpr (PLAIN) {
                             const float k = sd.kx[s];
-#pragma unroll
-                            for (int e = 0; e < kVEC; ++e)
-                                o[e] = euler_cell_iso(cen[s][e], xm[e], xp[e], yv[e], yw[e],
-                                                      zv[e], zw[e], k, inc[s][e]);
+                            euler4_iso(cen[s], xm, xp, yv, yw, zv, zw, k, inc[s], o);
                         } else {
                             species_core(sd, s, cen[s], xm, xp, yv, yw, zv, zw, inc[s], cx,
                                          src_here, px, xs, o);

@@ -2,8 +2,7 @@
 // 19-point Laplacian of eqs. (3)-(4), for the models without Cahn-Hilliard
 // (sm_103a).
 //
-// Work items, thread layout and copies follow the one-step 7-point kernel
-// (rd_step1_kernel): one thread per 4-cell vector of a 64 x TY tile plus one
+// Work items are those of the 7-point kernels: one thread per 4-cell vector of a 64 x TY tile plus one
 // halo warp, planes of the current state copied into a shared-memory ring
 // by per-thread cp.async several planes ahead, one barrier per plane.  What
 // differs:

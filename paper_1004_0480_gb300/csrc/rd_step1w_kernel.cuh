@@ -1,9 +1,10 @@
 // rd_step1w_kernel.cuh -- the one-step 7-point kernel with 8 cells per
 // thread (tile_q = 8 in rd_tuning), for the models without Cahn-Hilliard.
 //
-// The work items, the 64-cell tile width, the 6-slot cp.async ring of
-// planes, the halo warp and the boundary rules are those of rd_step1_kernel
-// (rd_step_kernel.cuh); what differs:
+// The work items and the 64-cell tile width are those of rd_march_kernel;
+// planes arrive in a 6-slot cp.async ring five copy groups ahead, with one
+// halo warp fetching the tile's halo, zero-flux ghosts copied in as face
+// values at distance one.
 //
 //  * Each compute thread owns 8 consecutive cells of a row: a tile row is 8
 //    threads, a warp 4 rows.  Its plane copies are 16 bytes for bfloat16
@@ -151,7 +152,7 @@ template <class A> __device__ __forceinline__ const float (&chalf4(const A& v, i
     return *reinterpret_cast<const float(*)[4]>(&v[4 * h]);
 }
 
-// PLAIN, W3: as rd_step1_kernel.  Tile heights are multiples of 4.
+// PLAIN, W3: as rd_march_kernel.  Tile heights are multiples of 4.
 template <class M, class ST, bool ONE, bool PLAIN, bool W3>
 __global__ void __launch_bounds__(kMaxThreads, 1)
 rd_step1w_kernel(const __grid_constant__ LaunchArgs a) {
@@ -242,7 +243,7 @@ rd_step1w_kernel(const __grid_constant__ LaunchArgs a) {
         if constexpr (W3) wind3d(sd, lin, local, cy, cz);
         __syncthreads();   // halo descriptors written
 
-        // ---- the march (as rd_step1_kernel)
+        // ---- the march: plane nld is fetched P planes ahead into slot sl
         int nld = z0 - 1;
         int zld = pz ? wrapi(nld, nz) : nld;
         auto issue = [&](int sl) {
@@ -318,13 +319,15 @@ rd_step1w_kernel(const __grid_constant__ LaunchArgs a) {
                     // reaction on the half's 4 cells
                     float inc[S][kVEC];
 #pragma unroll
-                    for (int e = 0; e < kVEC; ++e) {
-                        float cv[S], iv[S];
+                    for (int h2 = 0; h2 < 2; ++h2) {
+                        float2 cv[S], iv[S];
 #pragma unroll
-                        for (int s = 0; s < S; ++s) cv[s] = own_0[s][4 * h + e];
+                        for (int s = 0; s < S; ++s)
+                            cv[s] = make_float2(own_0[s][4 * h + 2 * h2],
+                                                own_0[s][4 * h + 2 * h2 + 1]);
                         M::react(sd, cv, iv);
 #pragma unroll
-                        for (int s = 0; s < S; ++s) inc[s][e] = iv[s];
+                        for (int s = 0; s < S; ++s) set_pair(inc[s], h2, iv[s]);
                     }
 #pragma unroll
                     for (int s = 0; s < S; ++s) {
@@ -343,10 +346,7 @@ rd_step1w_kernel(const __grid_constant__ LaunchArgs a) {
                         }
                         if constexpr (PLAIN) {
                             const float k = sd.kx[s];
-#pragma unroll
-                            for (int e = 0; e < kVEC; ++e)
-                                o[e] = euler_cell_iso(cen[e], xm[e], xp[e], ym[e], yp[e], zm[e],
-                                                      zp[e], k, inc[s][e]);
+                            euler4_iso(cen, xm, xp, ym, yp, zm, zp, k, inc[s], o);
                         } else {
                             species_core(sd, s, cen, xm, xp, ym, yp, zm, zp, inc[s], cx, src_here,
                                          px, xs + 4 * h, o, cy, cz);

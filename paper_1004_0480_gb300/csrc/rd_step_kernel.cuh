@@ -1,10 +1,11 @@
 // rd_step_kernel.cuh -- the fused forward-Euler step kernels (sm_103a).
 //
-// Three kernels share the per-cell update functions below, so every launch
-// shape gives the same bits: rd_step_kernel (T steps per launch, described
-// here), rd_step1_kernel (one step per launch, models without
-// Cahn-Hilliard) and rd_stepch_kernel (one step per launch, the front
-// model); the last two are described where they are defined.
+// The kernels share the per-cell update functions below, so every launch
+// shape gives the same bits: rd_step_kernel (T steps per launch, any tile
+// height, described here), rd_march_kernel (one or two steps per launch, even
+// heights, models without Cahn-Hilliard), rd_step1w_kernel (one step, 8 cells
+// per thread) and rd_stepch_kernel (one step, the Cahn-Hilliard models); the
+// others are described where they are defined.
 //
 // rd_step_kernel: one launch advances T steps of eq. (5) for every species
 // of every work item.  A work item is an x-y tile of 64 x TY cells and a chunk of z planes
@@ -44,10 +45,10 @@
 
 #include "rd_debug.cuh"
 #include "rd_internal.h"
+#include "rd_pack.cuh"
 
 namespace rdk {
 
-constexpr int kVEC = 4;               // cells per thread position (x)
 constexpr int kNQ = kTileQ + 2;       // vector positions per row incl. halo
 constexpr int kRW = kNQ * kVEC;       // elements per shared-memory row
 
@@ -164,8 +165,9 @@ __device__ __forceinline__ float courant_at(const InstDesc& sd, const float* tab
 struct MDiffusion {
     static constexpr int S = 1;
     static constexpr bool CH = false;
-    __device__ __forceinline__ static void react(const InstDesc&, const float*, float* inc) {
-        inc[0] = 0.0f;
+    template <class V>
+    __device__ __forceinline__ static void react(const InstDesc&, const V*, V* inc) {
+        inc[0] = vset<V>(0.0f);
     }
 };
 
@@ -174,13 +176,14 @@ struct MDiffusion {
 struct MBrusselator {
     static constexpr int S = 2;
     static constexpr bool CH = false;
-    __device__ __forceinline__ static void react(const InstDesc& d, const float* c, float* inc) {
-        const float u = c[0], v = c[1];
-        const float uuv = __fmul_rn(__fmul_rn(u, u), v);
-        const float f = __fadd_rn(__fmaf_rn(-d.p[1], u, d.p[0]), uuv);
-        const float g = __fsub_rn(__fmul_rn(d.p[2], u), uuv);
-        inc[0] = __fmul_rn(d.dt, f);
-        inc[1] = __fmul_rn(d.dt, g);
+    template <class V>
+    __device__ __forceinline__ static void react(const InstDesc& d, const V* c, V* inc) {
+        const V u = c[0], v = c[1];
+        const V uuv = vmul_rounded(vmul(u, u), v);
+        const V f = vadd(vfma(vset<V>(-d.p[1]), u, vset<V>(d.p[0])), uuv);
+        const V g = vsub(vmul_rounded(vset<V>(d.p[2]), u), uuv);
+        inc[0] = vmul(vset<V>(d.dt), f);
+        inc[1] = vmul(vset<V>(d.dt), g);
     }
 };
 
@@ -189,12 +192,13 @@ struct MBrusselator {
 struct MAir {
     static constexpr int S = 3;
     static constexpr bool CH = false;
-    __device__ __forceinline__ static void react(const InstDesc& d, const float* c, float* inc) {
-        const float ph = __fmul_rn(d.p[0], c[1]);
-        const float ti = __fmul_rn(__fmul_rn(d.p[1], c[0]), c[2]);
-        const float net = __fmul_rn(d.dt, __fsub_rn(ph, ti));
+    template <class V>
+    __device__ __forceinline__ static void react(const InstDesc& d, const V* c, V* inc) {
+        const V ph = vmul_rounded(vset<V>(d.p[0]), c[1]);
+        const V ti = vmul_rounded(vmul(vset<V>(d.p[1]), c[0]), c[2]);
+        const V net = vmul(vset<V>(d.dt), vsub(ph, ti));
         inc[0] = net;
-        inc[1] = -net;
+        inc[1] = vneg(net);
         inc[2] = net;
     }
 };
@@ -205,34 +209,22 @@ struct MAir {
 // c += p[1] Lap_h mu + dt R_c, with no Fickian term for c (the biharmonic
 // as "Laplacian, boundary rule, Laplacian", Section 4.1).
 
-// mu from g(c) and the 6 neighbours of c
-__device__ __forceinline__ float ch_mu(float g, float pk, float c, float xm, float xp, float ym,
-                                       float yp, float zm, float zp) {
-    const float s6 = __fadd_rn(__fadd_rn(__fadd_rn(xm, xp), __fadd_rn(ym, yp)), __fadd_rn(zm, zp));
-    const float lap = __fmaf_rn(-6.0f, c, s6);
-    return __fmaf_rn(-pk, lap, g);
-}
-
 // Front a + b -> c with Cahn-Hilliard c.
 // p[0] = dt k, p[1] = dt M / h^2, p[2] = kappa / h^2.
 struct MChFront {
     static constexpr int S = 3;
     static constexpr bool CH = true;
-    __device__ __forceinline__ static void react(const InstDesc& d, const float* c, float* inc) {
-        const float q = __fmul_rn(__fmul_rn(d.p[0], c[0]), c[1]);
-        inc[0] = -q;
-        inc[1] = -q;
+    template <class V>
+    __device__ __forceinline__ static void react(const InstDesc& d, const V* c, V* inc) {
+        const V q = vmul(vmul(vset<V>(d.p[0]), c[0]), c[1]);
+        inc[0] = vneg(q);
+        inc[1] = vneg(q);
         inc[2] = q;
     }
     // g(c) = f'(c) = 2c(c-1)(2c-1), the derivative of the double well
-    __device__ __forceinline__ static float g(const InstDesc&, float c) {
-        const float c2 = __fadd_rn(c, c);
-        return __fmul_rn(__fmul_rn(c2, __fsub_rn(c, 1.0f)), __fsub_rn(c2, 1.0f));
-    }
-    // mu = f'(c) - (kappa/h^2) (sum of 6 neighbours - 6 c)
-    __device__ __forceinline__ static float mu(const InstDesc& d, float c, float xm, float xp,
-                                               float ym, float yp, float zm, float zp) {
-        return ch_mu(g(d, c), d.p[2], c, xm, xp, ym, yp, zm, zp);
+    template <class V> __device__ __forceinline__ static V g(const InstDesc&, V c) {
+        const V c2 = vadd(c, c);
+        return vmul(vmul(c2, vadd(c, vset<V>(-1.0f))), vadd(c2, vset<V>(-1.0f)));
     }
 };
 
@@ -244,45 +236,130 @@ struct MChFront {
 struct MChTable1 {
     static constexpr int S = 3;
     static constexpr bool CH = true;
-    __device__ __forceinline__ static void react(const InstDesc& d, const float* c, float* inc) {
-        const float q1 = __fmul_rn(__fmul_rn(d.p[0], c[0]), c[1]);
-        const float q2 = __fmul_rn(__fmul_rn(d.p[3], c[0]), c[2]);
-        inc[0] = -__fadd_rn(q1, q2);
-        inc[1] = -q1;
-        inc[2] = __fsub_rn(q1, q2);
+    template <class V>
+    __device__ __forceinline__ static void react(const InstDesc& d, const V* c, V* inc) {
+        const V q1 = vmul_rounded(vmul(vset<V>(d.p[0]), c[0]), c[1]);
+        const V q2 = vmul_rounded(vmul(vset<V>(d.p[3]), c[0]), c[2]);
+        inc[0] = vneg(vadd(q1, q2));
+        inc[1] = vneg(q1);
+        inc[2] = vsub(q1, q2);
     }
     // g(c) = eps c - gamma c^3
-    __device__ __forceinline__ static float g(const InstDesc& d, float c) {
-        return __fmul_rn(c, __fmaf_rn(-d.p[5], __fmul_rn(c, c), d.p[4]));
-    }
-    __device__ __forceinline__ static float mu(const InstDesc& d, float c, float xm, float xp,
-                                               float ym, float yp, float zm, float zp) {
-        return ch_mu(g(d, c), d.p[2], c, xm, xp, ym, yp, zm, zp);
+    template <class V> __device__ __forceinline__ static V g(const InstDesc& d, V c) {
+        return vmul(c, vfma(vset<V>(-d.p[5]), vmul(c, c), vset<V>(d.p[4])));
     }
 };
 
-// One cell of eq. (5) for a species with Fickian transport:
-// c + inc + sum_a k_a (c[-1] + c[+1] - 2c), k_a = D_a dt / h^2.
-__device__ __forceinline__ float euler_cell(float c, float xm, float xp, float ym, float yp,
-                                            float zm, float zp, float kx, float ky, float kz,
-                                            float inc) {
-    const float c2 = __fadd_rn(c, c);
-    const float lx = __fsub_rn(__fadd_rn(xm, xp), c2);
-    const float ly = __fsub_rn(__fadd_rn(ym, yp), c2);
-    const float lz = __fsub_rn(__fadd_rn(zm, zp), c2);
-    inc = __fmaf_rn(kz, lz, inc);
-    inc = __fmaf_rn(ky, ly, inc);
-    inc = __fmaf_rn(kx, lx, inc);
-    return __fadd_rn(c, inc);
+// dt R_s(c) of the thread's 4 cells
+template <class M, int S>
+__device__ __forceinline__ void react4(const InstDesc& d, const float (&c)[S][kVEC],
+                                       float (&inc)[S][kVEC]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float2 cv[S], iv[S];
+#pragma unroll
+        for (int s = 0; s < S; ++s) cv[s] = pair_of(c[s], h);
+        M::react(d, cv, iv);
+#pragma unroll
+        for (int s = 0; s < S; ++s) set_pair(inc[s], h, iv[s]);
+    }
 }
 
-// Same for equal diffusivities on the three axes (k = D dt / h^2):
+// One cell (or pair) of eq. (5) for a species with Fickian transport:
+// c + inc + sum_a k_a (c[-1] + c[+1] - 2c), k_a = D_a dt / h^2; sx, sy, sz
+// are the sums of the two neighbours along each axis.
+template <class V>
+__device__ __forceinline__ V euler_cell(V c, V sx, V sy, V sz, float kx, float ky, float kz,
+                                        V inc) {
+    const V c2 = vadd(c, c);
+    inc = vfma(vset<V>(kz), vsub(sz, c2), inc);
+    inc = vfma(vset<V>(ky), vsub(sy, c2), inc);
+    inc = vfma(vset<V>(kx), vsub(sx, c2), inc);
+    return vadd(c, inc);
+}
+
+// Sum of the 6 neighbours - 6 c
+template <class V> __device__ __forceinline__ V lap7_cell(V c, V sx, V sy, V sz) {
+    return vfma(vset<V>(-6.0f), c, vadd(vadd(sx, sy), sz));
+}
+
+// euler_cell for equal diffusivities on the three axes (k = D dt / h^2):
 // c + inc + k (sum of the 6 neighbours - 6 c).
-__device__ __forceinline__ float euler_cell_iso(float c, float xm, float xp, float ym, float yp,
-                                                float zm, float zp, float k, float inc) {
-    const float s6 = __fadd_rn(__fadd_rn(__fadd_rn(xm, xp), __fadd_rn(ym, yp)), __fadd_rn(zm, zp));
-    const float lap = __fmaf_rn(-6.0f, c, s6);
-    return __fadd_rn(c, __fmaf_rn(k, lap, inc));
+template <class V>
+__device__ __forceinline__ V euler_cell_iso(V c, V sx, V sy, V sz, float k, V inc) {
+    return vadd(c, vfma(vset<V>(k), lap7_cell(c, sx, sy, sz), inc));
+}
+
+// The neighbour sums of the thread's cells 2h, 2h + 1.  The x neighbours of
+// a pair are no aligned pair of registers, so that sum is taken cell by cell.
+__device__ __forceinline__ float2 xsum_of(const float (&xm)[kVEC], const float (&xp)[kVEC],
+                                          int h) {
+    return make_float2(__fadd_rn(xm[2 * h], xp[2 * h]), __fadd_rn(xm[2 * h + 1], xp[2 * h + 1]));
+}
+
+// 4 cells of euler_cell_iso
+__device__ __forceinline__ void euler4_iso(const float (&c)[kVEC], const float (&xm)[kVEC],
+                                           const float (&xp)[kVEC], const float (&ym)[kVEC],
+                                           const float (&yp)[kVEC], const float (&zm)[kVEC],
+                                           const float (&zp)[kVEC], float k,
+                                           const float (&inc)[kVEC], float (&o)[kVEC]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        set_pair(o, h, euler_cell_iso(pair_of(c, h), xsum_of(xm, xp, h),
+                                      vadd(pair_of(ym, h), pair_of(yp, h)),
+                                      vadd(pair_of(zm, h), pair_of(zp, h)), k, pair_of(inc, h)));
+}
+
+// 4 cells of a species with any diffusivities: euler_cell_iso where they are
+// equal, else euler_cell
+__device__ __forceinline__ void euler4(const float (&c)[kVEC], const float (&xm)[kVEC],
+                                       const float (&xp)[kVEC], const float (&ym)[kVEC],
+                                       const float (&yp)[kVEC], const float (&zm)[kVEC],
+                                       const float (&zp)[kVEC], float kx, float ky, float kz,
+                                       const float (&inc)[kVEC], float (&o)[kVEC]) {
+    if (kx == ky && kx == kz) {
+        euler4_iso(c, xm, xp, ym, yp, zm, zp, kx, inc, o);
+        return;
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        set_pair(o, h, euler_cell(pair_of(c, h), xsum_of(xm, xp, h),
+                                  vadd(pair_of(ym, h), pair_of(yp, h)),
+                                  vadd(pair_of(zm, h), pair_of(zp, h)), kx, ky, kz,
+                                  pair_of(inc, h)));
+}
+
+// mu = g(c) - p[2] (sum of 6 neighbours - 6 c) of the thread's 4 cells
+template <class M>
+__device__ __forceinline__ void mu4(const InstDesc& d, const float (&c)[kVEC],
+                                    const float (&xm)[kVEC], const float (&xp)[kVEC],
+                                    const float (&ym)[kVEC], const float (&yp)[kVEC],
+                                    const float (&zm)[kVEC], const float (&zp)[kVEC],
+                                    float (&mu)[kVEC]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const float2 cc = pair_of(c, h);
+        const float2 lap = lap7_cell(cc, xsum_of(xm, xp, h),
+                                     vadd(pair_of(ym, h), pair_of(yp, h)),
+                                     vadd(pair_of(zm, h), pair_of(zp, h)));
+        set_pair(mu, h, vfma(vset<float2>(-d.p[2]), lap, M::g(d, cc)));
+    }
+}
+
+// c + inc + pm (sum of the 6 neighbours of mu - 6 mu): the Cahn-Hilliard
+// species' update on 4 cells, pm = p[1]
+__device__ __forceinline__ void euler4_ch(float pm, const float (&c)[kVEC], const float (&m)[kVEC],
+                                          const float (&xm)[kVEC], const float (&xp)[kVEC],
+                                          const float (&ym)[kVEC], const float (&yp)[kVEC],
+                                          const float (&zm)[kVEC], const float (&zp)[kVEC],
+                                          const float (&inc)[kVEC], float (&o)[kVEC]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const float2 lap = lap7_cell(pair_of(m, h), xsum_of(xm, xp, h),
+                                     vadd(pair_of(ym, h), pair_of(yp, h)),
+                                     vadd(pair_of(zm, h), pair_of(zp, h)));
+        set_pair(o, h, vadd(pair_of(c, h), vfma(vset<float2>(pm), lap, pair_of(inc, h))));
+    }
 }
 
 // ------------------------------------------------------- shared-memory map
@@ -473,10 +550,14 @@ __device__ __forceinline__ void upwind_axis(float cu, const float (&c)[kVEC],
                                             float (&in)[kVEC]) {
     if (cu > 0.0f) {
 #pragma unroll
-        for (int e = 0; e < kVEC; ++e) in[e] = __fmaf_rn(-cu, __fsub_rn(c[e], cm[e]), in[e]);
+        for (int h = 0; h < 2; ++h)
+            set_pair(in, h, vfma(vset<float2>(-cu), vsub(pair_of(c, h), pair_of(cm, h)),
+                                 pair_of(in, h)));
     } else if (cu < 0.0f) {
 #pragma unroll
-        for (int e = 0; e < kVEC; ++e) in[e] = __fmaf_rn(-cu, __fsub_rn(cp[e], c[e]), in[e]);
+        for (int h = 0; h < 2; ++h)
+            set_pair(in, h, vfma(vset<float2>(-cu), vsub(pair_of(cp, h), pair_of(c, h)),
+                                 pair_of(in, h)));
     }
 }
 
@@ -510,7 +591,6 @@ __device__ __forceinline__ void species_core(const InstDesc& sd, int s, const fl
                                              float cz = 0.0f) {
     const float kx = sd.kx[s], ky = sd.ky[s], kz = sd.kz[s];
     const bool src_s = src_here && s == sd.src_s;
-    const bool iso = kx == ky && kx == kz;
     // every test below is uniform over the 4 cells: taken once, not per cell
     float in[kVEC];
 #pragma unroll
@@ -520,7 +600,8 @@ __device__ __forceinline__ void species_core(const InstDesc& sd, int s, const fl
         for (int e = 0; e < kVEC; ++e)
             if ((px ? wrapi(xs + e, sd.nx) : xs + e) == sd.src_x) in[e] = __fadd_rn(in[e], sd.src_amt);
     }
-    // first-order upwind advection, Courant number cx = u dt / h
+    // first-order upwind advection, Courant number cx = u dt / h; the x
+    // differences cell by cell (see xsum_of)
     if (cx > 0.0f) {
 #pragma unroll
         for (int e = 0; e < kVEC; ++e) in[e] = __fmaf_rn(-cx, __fsub_rn(c[e], xm[e]), in[e]);
@@ -531,15 +612,7 @@ __device__ __forceinline__ void species_core(const InstDesc& sd, int s, const fl
     // the same along y and z (the 3-D wind of Table 1, row 4)
     upwind_axis(cy, c, ym, yp, in);
     upwind_axis(cz, c, zm, zp, in);
-    if (iso) {
-#pragma unroll
-        for (int e = 0; e < kVEC; ++e)
-            o[e] = euler_cell_iso(c[e], xm[e], xp[e], ym[e], yp[e], zm[e], zp[e], kx, in[e]);
-    } else {
-#pragma unroll
-        for (int e = 0; e < kVEC; ++e)
-            o[e] = euler_cell(c[e], xm[e], xp[e], ym[e], yp[e], zm[e], zp[e], kx, ky, kz, in[e]);
-    }
+    euler4(c, xm, xp, ym, yp, zm, zp, kx, ky, kz, in, o);
 }
 
 // species_core followed by the held layers
@@ -702,9 +775,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) rd_step_kernel(const __grid_co
                         gather7<ST>(state_plane(l - 1, 2, q), state_plane(l - 1, 2, qm),
                                     state_plane(l - 1, 2, qp), ps, c, xm, xp, ym, yp, zm, zp);
                         float mo[kVEC];
-#pragma unroll
-                        for (int e = 0; e < kVEC; ++e)
-                            mo[e] = M::mu(sd, c[e], xm[e], xp[e], ym[e], yp[e], zm[e], zp[e]);
+                        mu4<M>(sd, c, xm, xp, ym, yp, zm, zp, mo);
                         Store<float>::store(mu_plane(l, q) + ps.own, mo);
                         continue;
                     }
@@ -716,15 +787,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) rd_step_kernel(const __grid_co
                     float cen[S][kVEC];
 #pragma unroll
                     for (int s = 0; s < S; ++s) Store<ST>::load(state_plane(ls, s, q) + ps.own, cen[s]);
-#pragma unroll
-                    for (int e = 0; e < kVEC; ++e) {
-                        float cv[S], iv[S];
-#pragma unroll
-                        for (int s = 0; s < S; ++s) cv[s] = cen[s][e];
-                        M::react(sd, cv, iv);
-#pragma unroll
-                        for (int s = 0; s < S; ++s) inc[s][e] = iv[s];
-                    }
+                    react4<M>(sd, cen, inc);
                 }
                 const float cx = courant_at(sd, sd.courant, zw);
                 const bool src_here = src_col && zw == sd.src_z;
@@ -738,14 +801,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) rd_step_kernel(const __grid_co
                         gather7<float>(mu_plane(l - 1, q), mu_plane(l - 1, qm), mu_plane(l - 1, qp),
                                        ps, m0, mxm, mxp, mym, myp, mzm, mzp);
                         Store<ST>::load(state_plane(ls, 2, q) + ps.own, c);
-#pragma unroll
-                        for (int e = 0; e < kVEC; ++e) {
-                            const float s6 = __fadd_rn(
-                                __fadd_rn(__fadd_rn(mxm[e], mxp[e]), __fadd_rn(mym[e], myp[e])),
-                                __fadd_rn(mzm[e], mzp[e]));
-                            const float lap = __fmaf_rn(-6.0f, m0[e], s6);
-                            o[e] = __fadd_rn(c[e], __fmaf_rn(sd.p[1], lap, inc[s][e]));
-                        }
+                        euler4_ch(sd.p[1], c, m0, mxm, mxp, mym, myp, mzm, mzp, inc[s], o);
                     } else {
                         float c[kVEC], xm[kVEC], xp[kVEC], ym[kVEC], yp[kVEC], zm[kVEC], zp[kVEC];
                         gather7<ST>(state_plane(ls, s, q), state_plane(ls, s, qm),
@@ -771,29 +827,6 @@ __global__ void __launch_bounds__(kMaxThreads, 2) rd_step_kernel(const __grid_co
         __syncthreads();
     }
 }
-
-// ------------------------------------------------------ one-step kernel
-// The T = 1 path of the models without Cahn-Hilliard.  16 x TY compute
-// threads, one per 4-cell vector of a 64 x TY tile, plus one halo warp that
-// fetches the tile's halo (one row above and below, one vector left and
-// right; the 7-point stencil needs no corners).  Planes arrive in a 6-slot
-// shared-memory ring: while plane q is computed, planes q-1..q+1 are
-// resident and q+2..q+4 in flight (P = 5 copy groups ahead of q-1).  A
-// compute thread reads its own vector in planes q-1, q, q+1 and its four
-// neighbours in plane q.  The slot refilled at step q held plane q-2: its
-// neighbour reads ended two barriers earlier and its own-vector reads
-// precede the refill in the owner's program order, so one barrier per plane
-// suffices.  The halo warp runs its own copy loop with the same barriers.
-template <class M, class ST> struct Layout1 {
-    static constexpr int S = M::S;
-    static constexpr int RING = 6;
-    static constexpr int P = 5;
-    __host__ __device__ static int plane_elems(int ty) { return (ty + 2) * kRW + 2 * kVEC; }
-    __host__ __device__ static size_t total(int ty) {
-        return (size_t)RING * S * plane_elems(ty) * sizeof(ST) + 96 * sizeof(int4);
-    }
-    __host__ __device__ static int threads(int ty) { return kTileQ * ty + 32; }
-};
 
 // How one vector is fetched: 1 = one async copy, 2 = element by element
 // (wrapped x, or clamped x for a vector straddling a zero-flux face), 0 =
@@ -892,278 +925,66 @@ __device__ __forceinline__ float lds_one(const unsigned char* p) {
     return Store<ST>::get(reinterpret_cast<const ST*>(p));
 }
 
-// Zero-flux ghost cells are copied in as face values at distance one (rows,
-// planes, and vectors straddling the face), as the paper sets its boundary
-// layer before each step; a thread at an x face reads its x neighbour
-// beyond the face from its own vector (xface_offsets).  Every other
-// neighbour sits at a fixed offset from the thread's own vector.  An upwind
-// inflow face sees a zero gradient, and a held layer's ghost only feeds the
-// held cell's own update, which is replaced by its bc value, so this is
-// exact for every one-step problem.
-// PLAIN: no held layer, point source or wind, and every species isotropic;
-// the update then needs no per-plane or per-species branches.  W3: the
-// 3-D wind (upwind along y and z too; never with PLAIN).
-template <class M, class ST, bool ONE, int MINB, bool PLAIN, bool W3>
-__global__ void __launch_bounds__(kMaxThreads, MINB)
-rd_step1_kernel(const __grid_constant__ LaunchArgs a) {
-    using LY = Layout1<M, ST>;
-    constexpr int S = M::S;
-    constexpr int P = LY::P;
-    constexpr int RING = LY::RING;
-    constexpr int EB = (int)sizeof(ST);
-    constexpr int RWB = kRW * EB;                            // bytes per shared row
-
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ InstDesc sdm;
-    __shared__ int s_inst;
-    __shared__ long long s_item;
-
-    const int tid = threadIdx.x;
-    const int TY = a.ty;
-    const int PEB = LY::plane_elems(TY) * EB;                // bytes per species plane
-    const int SLOTB = S * PEB;                               // bytes per ring slot
-    unsigned char* const ring = smem + kVEC * EB;            // slot 0, species 0
-    int4* const hfetch = reinterpret_cast<int4*>(smem + RING * SLOTB);
-    const int ncomp = kTileQ * TY;
-    const bool halo_warp = tid >= ncomp;
-    const int r = tid / kTileQ;
-    const int v = tid - r * kTileQ;
-    const int own_b = ((r + 1) * kRW + (v + 1) * kVEC) * EB;
-
-    int cur_inst = -1;
-    if (tid == 0) s_inst = 0;
-    for (long long item = first_item<ONE>(a, s_item); item < a.nitems;
-         item = next_item<ONE>(a, item, s_item)) {
-        if constexpr (!ONE) load_desc(a, item, sdm, s_inst, cur_inst);
-        const InstDesc& sd = desc_of<ONE>(a, sdm);
-        if (member_done<ONE>(a, sd)) continue;   // block-uniform
-
-        const int nx = sd.nx, ny = sd.ny, nz = sd.nz, pitch = sd.pitch;
-        const bool px = sd.per_x, py = sd.per_y, pz = sd.per_z;
-        // element-wise copies: periodic x with nx % 4 != 0, and zero-flux x faces
-        const bool elems = sd.wrap_elems || !sd.per_x;
-        const long long local = item - sd.item_begin;
-        const int txi = (int)(local % sd.ntx);
-        const int tyi = (int)((local / sd.ntx) % sd.nty);
-        const int zc = (int)(local / ((long long)sd.ntx * sd.nty));
-        const int x0 = txi * kTileQ * kVEC, y0 = tyi * TY;
-        const int z0 = zc * sd.zchunk;
-        const int z1 = min(z0 + sd.zchunk, nz);
-        const int lin = sd.par ^ a.parity;
-        const ST* const gin = reinterpret_cast<const ST*>(sd.base[lin][0]);
-        ST* const gout = reinterpret_cast<ST*>(sd.base[lin ^ 1][0]);
-        // the fields of one instance and time level are evenly spaced
-        const long long fstride = S > 1 ? reinterpret_cast<const ST*>(sd.base[lin][1]) - gin : 0;
-        const long long plane = sd.plane;
-
-        // ---- halo lanes: up to three halo vectors each, described in shared
-        // memory (2 TY side vectors, then 2 x 16 row vectors)
-        if (halo_warp) {
-            const int hl = tid - ncomp;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const int j = hl + 32 * k;
-                Fetch f{0, 0, 0, 0};
-                if (j < 2 * TY) {
-                    const int hr = j >> 1;
-                    const bool right = j & 1;
-                    const int xh = right ? x0 + kTileQ * kVEC : x0 - kVEC;
-                    f = make_fetch<ST>(y0 + hr, xh, nx, ny, pitch, px, py,
-                                       (hr + 1) * kRW + (right ? kNQ - 1 : 0) * kVEC, true);
-                } else if (j < 2 * TY + 2 * kTileQ) {
-                    const int jj = j - 2 * TY;
-                    const bool bottom = jj >= kTileQ;
-                    const int hv = jj - (bottom ? kTileQ : 0);
-                    f = make_fetch<ST>(bottom ? y0 + TY : y0 - 1, x0 + hv * kVEC, nx, ny, pitch, px,
-                                       py, (bottom ? TY + 1 : 0) * kRW + (hv + 1) * kVEC, true);
-                }
-                if (RD_DBG_SHARED(hfetch + j, 16, kSiteHaloDesc))
-                    hfetch[j] = make_int4(f.mode, f.goff, f.soff, f.xs);
-            }
-        }
-        // ---- compute threads: own vector and its neighbours
-        const int y = y0 + r;
-        const int xs = x0 + v * kVEC;
-        const bool computes = !halo_warp && y < ny && xs < nx;
-        const bool src_col = sd.src_s >= 0 && (py ? wrapi(y, ny) : y) == sd.src_y;
-        const unsigned xyf = xy_faces(xs, y, nx, ny);
-        const Fetch fo = halo_warp ? Fetch{0, 0, 0, 0}
-                                   : make_fetch<ST>(y, xs, nx, ny, pitch, px, py, own_b / EB, true);
-        int loff, roff;                           // x neighbours beside the own vector
-        xface_offsets<ST>(xs, nx, px, loff, roff);
-        float cy = 0.0f, cz = 0.0f;               // 3-D wind
-        if constexpr (W3) wind3d(sd, lin, local, cy, cz);
-        __syncthreads();   // halo descriptors written
-
-        // ---- the march: plane nld is fetched P planes ahead into slot sl;
-        // plane z0 - 1 goes to slot 0, plane q to slot (q - z0 + 1) mod RING
-        int nld = z0 - 1;
-        int zld = pz ? wrapi(nld, nz) : nld;      // plane index the copy reads
-        auto issue = [&](int sl) {
-            // zero-flux z: the face plane is copied in as the ghost plane
-            const bool in_z = pz || (nld >= 0 && nld < nz);
-            if (nld <= z1) {
-                const int zs = in_z ? zld : (nld < 0 ? 0 : nz - 1);
-                const ST* gld = gin + (long long)zs * plane;
-                unsigned char* buf = ring + sl * SLOTB;
-                if (halo_warp) {
-                    const int hl = tid - ncomp;
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        int4 h = make_int4(0, 0, 0, 0);
-                        if (RD_DBG_SHARED(hfetch + hl + 32 * k, 16, kSiteHaloDesc))
-                            h = hfetch[hl + 32 * k];
-                        fetch_all<ST, S>(Fetch{h.x, h.y, h.z, h.w}, buf, PEB, gld, fstride, nx,
-                                         elems, px, sd);
-                    }
-                } else {
-                    fetch_all<ST, S>(fo, buf, PEB, gld, fstride, nx, elems, px, sd);
-                }
-            }
-            ++nld;
-            if (!pz) zld = nld;
-            else if (++zld == nz) zld = 0;
-            cp_async_commit();
-        };
-#pragma unroll 1
-        for (int j = 0; j < P; ++j) issue(j);
-        int zq = pz ? wrapi(z0, nz) : z0;       // wrapped index of plane q
-        ST* gst = gout + (long long)z0 * plane + (long long)y * pitch + xs;
-        const float* courant = sd.courant;
-        int sc = 1;                               // ring slot of plane q
-        // own vectors of planes q-1 and q, carried down the march
-        float own_m[S][kVEC], own_0[S][kVEC];
-#pragma unroll 1
-        for (int q = z0; q < z1; ++q) {
-            const int sm = sc == 0 ? RING - 1 : sc - 1;
-            const int sp = sc == RING - 1 ? 0 : sc + 1;
-            // planes up to q + 1 must have landed: of the P + (q - z0 + 1)
-            // groups issued so far, all but the newest P - 2
-            issue(sc >= RING - P + 1 ? sc + P - 1 - RING : sc + P - 1);
-            cp_async_wait<P - 2>();
-            __syncthreads();
-            if (!halo_warp) {
-                // every neighbour at a fixed offset; ghosts were copied in
-                const unsigned char* Pc = ring + sc * SLOTB + own_b;
-                const unsigned char* Pp = ring + sp * SLOTB + own_b;
-                if (q == z0) {
-                    const unsigned char* Pm = ring + sm * SLOTB + own_b;
-#pragma unroll
-                    for (int s = 0; s < S; ++s) {
-                        lds_vec<ST>(Pm + s * PEB, own_m[s]);
-                        lds_vec<ST>(Pc + s * PEB, own_0[s]);
-                    }
-                }
-                float own_p[S][kVEC], inc[S][kVEC];
-#pragma unroll
-                for (int s = 0; s < S; ++s) lds_vec<ST>(Pp + s * PEB, own_p[s]);
-                auto& cen = own_0;
-#pragma unroll
-                for (int e = 0; e < kVEC; ++e) {
-                    float cv[S], iv[S];
-#pragma unroll
-                    for (int s = 0; s < S; ++s) cv[s] = cen[s][e];
-                    M::react(sd, cv, iv);
-#pragma unroll
-                    for (int s = 0; s < S; ++s) inc[s][e] = iv[s];
-                }
-                const float cx = courant_at(sd, courant, zq);
-                const bool src_here = src_col && zq == sd.src_z;
-                const unsigned faces = xyf | z_faces(q, nz);
-#pragma unroll
-                for (int s = 0; s < S; ++s) {
-                    const unsigned char* Ps = Pc + s * PEB;
-                    float xm[kVEC], xp[kVEC], ym[kVEC], yp[kVEC], o[kVEC];
-                    const float (&zm)[kVEC] = own_m[s];
-                    const float (&zp)[kVEC] = own_p[s];
-                    lds_vec<ST>(Ps - RWB, ym);
-                    lds_vec<ST>(Ps + RWB, yp);
-                    const float left = lds_one<ST>(Ps + loff);
-                    const float right = lds_one<ST>(Ps + roff);
-#pragma unroll
-                    for (int e = 0; e < kVEC; ++e) {
-                        xm[e] = e ? cen[s][e - 1] : left;
-                        xp[e] = (e < kVEC - 1) ? cen[s][e + 1] : right;
-                    }
-                    if constexpr (PLAIN) {
-                        // the same arithmetic species_update takes for this case
-                        const float k = sd.kx[s];
-#pragma unroll
-                        for (int e = 0; e < kVEC; ++e)
-                            o[e] = euler_cell_iso(cen[s][e], xm[e], xp[e], ym[e], yp[e], zm[e],
-                                                  zp[e], k, inc[s][e]);
-                    } else {
-                        species_core(sd, s, cen[s], xm, xp, ym, yp, zm, zp, inc[s], cx, src_here,
-                                     px, xs, o, cy, cz);
-                        held_layers_at(sd, s, faces, xs, y, q, o);
-                    }
-                    if (computes &&
-                        RD_DBG_GLOBAL(sd, gst + s * fstride, 4 * (int)sizeof(ST), kSiteStateStore))
-                        Store<ST>::store(gst + s * fstride, o);
-                }
-#pragma unroll
-                for (int s = 0; s < S; ++s)
-#pragma unroll
-                    for (int e = 0; e < kVEC; ++e) {
-                        own_m[s][e] = own_0[s][e];
-                        own_0[s][e] = own_p[s][e];
-                    }
-            }
-            gst += plane;
-            sc = sc == RING - 1 ? 0 : sc + 1;
-            if (!pz) zq = q + 1;
-            else if (++zq == nz) zq = 0;
-        }
-        cp_async_wait<0>();
-        __syncthreads();
-    }
-}
 }  // namespace rdk
 
 #include "rd_step1w_kernel.cuh"
 #include "rd_stepch_kernel.cuh"
+#include "rd_march_kernel.cuh"
 
 namespace rdk {
+
+// Whether T steps per launch at tile height ty run the two-step kernel
+// (whole inner warps: even heights; its CTA size); else the multi-level one.
+template <class M, class ST> constexpr bool two_step(int T, int ty) {
+    return T == 2 && !M::CH && !(ty & 1) && LayoutM<M, ST, 2>::threads(ty) <= kMaxThreads;
+}
 
 // Launch helper used by the per-model translation units.
 template <class M, class ST, int T, bool ONE>
 cudaError_t launch_one(const LaunchArgs& a, int grid, size_t smem, cudaStream_t st, int* occ) {
-    // the one-step kernel needs an even tile height (16 ty compute threads,
-    // then a whole halo warp); an odd one -- the last launch of a call whose
-    // tuning steps 2 or 3 per launch -- runs the multi-level kernel at T = 1
-    const bool lean = (T == 1 && !M::CH) && !(a.ty & 1);
-    constexpr bool lean_ch = (T == 1 && M::CH);
-    void (*k)(const LaunchArgs);
-    // 8 cells per thread: the one-step kernel of rd_step1w_kernel.cuh
-    const bool wide = lean && a.vw == 8;
-    if constexpr (lean_ch) {
+    void (*k)(const LaunchArgs) = nullptr;
+    int threads = 0;
+    // which kernel, and its slot in ``configured`` below
+    int variant = 0;
+    if constexpr (T == 1 && M::CH) {
         k = a.plain ? rd_stepch_kernel<M, ST, ONE, true> : rd_stepch_kernel<M, ST, ONE, false>;
-    } else if (wide) {
-        k = a.plain  ? rd_step1w_kernel<M, ST, ONE, true, false>
-            : a.wind3 ? rd_step1w_kernel<M, ST, ONE, false, true>
-                      : rd_step1w_kernel<M, ST, ONE, false, false>;
-    } else if (lean) {
-        // register budget of the one-step kernel: 128 (regcap 0) or 64 (regcap 1)
-        if (a.plain)
-            k = a.regcap ? rd_step1_kernel<M, ST, ONE, 2, true, false>
-                         : rd_step1_kernel<M, ST, ONE, 1, true, false>;
-        else if (a.wind3)
-            k = a.regcap ? rd_step1_kernel<M, ST, ONE, 2, false, true>
-                         : rd_step1_kernel<M, ST, ONE, 1, false, true>;
-        else
-            k = a.regcap ? rd_step1_kernel<M, ST, ONE, 2, false, false>
-                         : rd_step1_kernel<M, ST, ONE, 1, false, false>;
+        threads = LayoutCH<ST>::threads(a.ty);
+        variant = a.plain ? 1 : 0;
+    } else if constexpr (T == 1) {
+        // the march kernel needs an even tile height (16 ty inner threads as
+        // whole warps); an odd one -- the last launch of a
+        // call whose tuning steps 2 or 3 per launch -- runs the multi-level
+        // kernel at T = 1
+        const bool lean = !(a.ty & 1);
+        if (lean && a.vw == 8) {   // 8 cells per thread (rd_step1w_kernel.cuh)
+            k = a.plain   ? rd_step1w_kernel<M, ST, ONE, true, false>
+                : a.wind3 ? rd_step1w_kernel<M, ST, ONE, false, true>
+                          : rd_step1w_kernel<M, ST, ONE, false, false>;
+            threads = Layout1w<M, ST>::threads(a.ty);
+            variant = a.plain ? 1 : a.wind3 ? 2 : 3;
+        } else if (lean) {
+            k = a.plain   ? rd_march_kernel<M, ST, 1, ONE, true, false>
+                : a.wind3 ? rd_march_kernel<M, ST, 1, ONE, false, true>
+                          : rd_march_kernel<M, ST, 1, ONE, false, false>;
+            threads = LayoutM<M, ST, 1>::threads(a.ty);
+            variant = a.plain ? 4 : a.wind3 ? 5 : 6;
+        } else {
+            k = rd_step_kernel<M, ST, T, ONE>;
+            threads = Layout<M, ST, T>::threads(a.ty);
+        }
     } else {
         k = rd_step_kernel<M, ST, T, ONE>;
+        threads = Layout<M, ST, T>::threads(a.ty);
+        if constexpr (T == 2 && !M::CH)
+            if (two_step<M, ST>(T, a.ty)) {
+                k = a.plain ? rd_march_kernel<M, ST, 2, ONE, true, false>
+                            : rd_march_kernel<M, ST, 2, ONE, false, false>;
+                threads = LayoutM<M, ST, 2>::threads(a.ty);
+                variant = a.plain ? 1 : 2;
+            }
     }
-    // dynamic shared memory granted so far, per kernel variant (4: the
-    // multi-level kernel at T = 1; 5, 6: the one-step kernel with 3-D wind;
-    // 7, 8, 9: the 8-cell kernel, plain, 3-D wind, general)
-    static size_t configured[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-    const int variant = wide ? (a.plain ? 7 : a.wind3 ? 8 : 9)
-                        : (T == 1 && !M::CH && !lean) ? 4
-                        : (lean && !a.plain && a.wind3) ? 5 + (a.regcap ? 1 : 0)
-                        : (lean && a.regcap ? 1 : 0) + ((lean || lean_ch) && a.plain ? 2 : 0);
+    // dynamic shared memory granted so far, per kernel variant
+    static size_t configured[7] = {0, 0, 0, 0, 0, 0, 0};
     size_t& conf = configured[variant];
     if (smem > conf) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1171,10 +992,6 @@ cudaError_t launch_one(const LaunchArgs& a, int grid, size_t smem, cudaStream_t 
         if (e != cudaSuccess) return e;
         conf = smem;
     }
-    const int threads = wide      ? Layout1w<M, ST>::threads(a.ty)
-                        : lean    ? Layout1<M, ST>::threads(a.ty)
-                        : lean_ch ? LayoutCH<ST>::threads(a.ty)
-                                  : Layout<M, ST, T>::threads(a.ty);
     if (threads > kMaxThreads) return cudaErrorInvalidConfiguration;
     if (occ) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, threads, smem);
     k<<<grid, threads, smem, st>>>(a);
@@ -1220,16 +1037,21 @@ size_t smem_for(int storage, int tsteps, int ty, int vw = 4) {
     if (storage == RD_STORE_F32) {
         switch (tsteps) {
         case 1: return M::CH ? LayoutCH<float>::total(ty)
-                             : (ty & 1) ? Layout<M, float, 1>::total(ty) : Layout1<M, float>::total(ty);
-        case 2: return Layout<M, float, 2>::total(ty);
+                             : (ty & 1) ? Layout<M, float, 1>::total(ty) : LayoutM<M, float, 1>::total(ty);
+        case 2: if constexpr (!M::CH)
+                    if (two_step<M, float>(2, ty)) return LayoutM<M, float, 2>::total(ty);
+                return Layout<M, float, 2>::total(ty);
         case 3: return Layout<M, float, 3>::total(ty);
         }
     } else {
         switch (tsteps) {
         case 1: return M::CH ? LayoutCH<__nv_bfloat16>::total(ty)
                              : (ty & 1) ? Layout<M, __nv_bfloat16, 1>::total(ty)
-                                        : Layout1<M, __nv_bfloat16>::total(ty);
-        case 2: return Layout<M, __nv_bfloat16, 2>::total(ty);
+                                        : LayoutM<M, __nv_bfloat16, 1>::total(ty);
+        case 2: if constexpr (!M::CH)
+                    if (two_step<M, __nv_bfloat16>(2, ty))
+                        return LayoutM<M, __nv_bfloat16, 2>::total(ty);
+                return Layout<M, __nv_bfloat16, 2>::total(ty);
         case 3: return Layout<M, __nv_bfloat16, 3>::total(ty);
         }
     }

@@ -267,7 +267,9 @@ rd_stepch_kernel(const __grid_constant__ LaunchArgs a) {
                 for (int e = 0; e < kVEC; ++e) {
                     const float xm = e ? c[e - 1] : left;
                     const float xp = (e < kVEC - 1) ? c[e + 1] : right;
-                    mu_p[e] = MC::mu(sd, c[e], xm, xp, ym[e], yp[e], zm[e], zp[e]);
+                    const float lap = lap7_cell(c[e], vadd(xm, xp), vadd(ym[e], yp[e]),
+                                                vadd(zm[e], zp[e]));
+                    mu_p[e] = vfma(-sd.p[2], lap, MC::g(sd, c[e]));
                 }
                 Store<float>::store(muring + ((p + 1) & 1) * PE + own, mu_p);
             }
@@ -313,8 +315,9 @@ rd_stepch_kernel(const __grid_constant__ LaunchArgs a) {
                         const float k = sd.kx[s];
 #pragma unroll
                         for (int e = 0; e < kVEC; ++e)
-                            o[e] = euler_cell_iso(cen[s][e], xm[e], xp[e], ym[e], yp[e], zm[e],
-                                                  zp[e], k, inc[s][e]);
+                            o[e] = euler_cell_iso(cen[s][e], vadd(xm[e], xp[e]),
+                                                  vadd(ym[e], yp[e]), vadd(zm[e], zp[e]), k,
+                                                  inc[s][e]);
                     } else {
                         species_core(sd, s, cen[s], xm, xp, ym, yp, zm, zp, inc[s], cx, src_here,
                                      px, xs, o);
