@@ -563,22 +563,28 @@ rd_tuning default_tuning(const rd_config& g) {
     return t;
 }
 
-// Cost of a plane of one work item, in microseconds: a + b x (tile rows
-// resident on the SM), fitted to sweeps of tile heights and z-chunks on a
-// GB300 (grids of 32^3 to 512^3, see rd_march_kernel.cuh for the rates).  An
-// SM marches the rows of its CTAs at one rate, so more CTAs or taller tiles
-// cost the same per row; what a small grid saves is planes per item.
+// Time an SM takes per plane of its work items, in microseconds:
+// a + a1 / (CTAs on it) + b x (tile rows on it), fitted to sweeps of tile
+// heights and z-chunks on a GB300 (grids of 32^3 to 512^3).  An SM marches
+// the rows of its CTAs at about one rate, so more CTAs or taller tiles cost
+// the same per row; what a small grid saves is planes per item.
 struct PlaneCost {
-    double a, b;
+    double a, a1, b;
 };
-PlaneCost plane_cost(int nspecies, int storage, int T) {
-    const bool h = storage == RD_STORE_BF16;
-    switch (nspecies) {
-    case 1: return T == 2 ? PlaneCost{0.20, 0.0135} : PlaneCost{0.17, 0.0085};
+PlaneCost plane_cost(const rd_config& g, int T) {
+    const bool h = g.storage == RD_STORE_BF16;
+    if (stencil_of(g) == 19) {   // Cahn-Hilliard: both launches of a step
+        if (is_ch(g.model)) return {1.05, 0.5, 0.0200};
+        return g.nspecies == 1   ? PlaneCost{0.49, 0.0, 0.0107}
+               : g.nspecies == 2 ? PlaneCost{0.0, 0.6, 0.0146}
+                                 : PlaneCost{0.0, 0.9, 0.0300};
+    }
+    switch (g.nspecies) {
+    case 1: return T == 2 ? PlaneCost{0.20, 0.0, 0.0135} : PlaneCost{0.17, 0.0, 0.0085};
     case 2:
-        if (h) return T == 2 ? PlaneCost{0.30, 0.0197} : PlaneCost{0.30, 0.0079};
-        return T == 2 ? PlaneCost{0.10, 0.0335} : PlaneCost{0.15, 0.0185};
-    default: return T == 2 ? PlaneCost{0.40, 0.0770} : PlaneCost{0.30, 0.0340};
+        if (h) return T == 2 ? PlaneCost{0.30, 0.0, 0.0220} : PlaneCost{0.30, 0.0, 0.0079};
+        return T == 2 ? PlaneCost{0.10, 0.0, 0.0335} : PlaneCost{0.15, 0.0, 0.0185};
+    default: return T == 2 ? PlaneCost{0.40, 0.0, 0.0770} : PlaneCost{0.30, 0.0, 0.0340};
     }
 }
 // launch gap and pipeline fill of a launch (replayed from a graph)
@@ -594,7 +600,8 @@ constexpr double kLaunchUs = 2.4;
 // launch gap does not decide.
 rd_tuning default_plan(const rd_config& g, const rd_tuning& t1, int maxT) {
     rd_tuning best = t1;
-    if (is_ch(g.model) || stencil_of(g) == 19) {   // no plan: the tuning as it is
+    const int sten = stencil_of(g);
+    if (is_ch(g.model) && sten == 7) {   // no plan: the tuning as it is
         best.tsteps = 0;
         return best;
     }
@@ -607,9 +614,13 @@ rd_tuning default_plan(const rd_config& g, const rd_tuning& t1, int maxT) {
             t.tile_y = ty;
             t.zchunk = 1;
             if (T > 2 || check_tuning(g, t) != RD_OK) continue;
-            const int occ = occupancy(g.model, g.storage, T, ty, 0, variant_code(g), 7);
+            const int occ = occupancy(g.model, g.storage, T, ty, 0, variant_code(g), sten);
             if (occ < 1) continue;
-            const PlaneCost pc = plane_cost(g.nspecies, g.storage, T);
+            const PlaneCost pc = plane_cost(g, T);
+            // an SM's time per plane with ``ctas`` work items on it
+            auto plane_us = [&](int ctas) {
+                return ctas ? pc.a + pc.a1 / ctas + pc.b * ctas * ty : 0.0;
+            };
             const long long cols = (long long)tiles(g.nx, kTileW) * tiles(g.ny, ty);
             const long long slots = (long long)occ * sms;
             int last = 0;
@@ -619,11 +630,10 @@ rd_tuning default_plan(const rd_config& g, const rd_tuning& t1, int maxT) {
                 last = zc;
                 const long long items = cols * tiles(g.nz, zc);
                 const long long full = items / slots, rest = items % slots;
-                const long long rows = tiles((int)rest, sms) * (long long)ty;
                 const double planes = zc + 2 * (T - 1) + 1;
                 const double us =
-                    planes * (full * (pc.a + pc.b * occ * ty) + (rest ? pc.a + pc.b * rows : 0.0));
-                const double cost = (kLaunchUs + us) / T;
+                    planes * (full * plane_us(occ) + plane_us(tiles((int)rest, sms)));
+                const double cost = (kLaunchUs * kernels_per_step(g) + us) / T;
                 if (best_cost < 0 || cost < best_cost) {
                     best_cost = cost;
                     best = t;
@@ -736,7 +746,7 @@ rd_status upload_desc(rd_ctx* c) {
     fill_desc(c, c->desc, c->tun);
     if (c->plan.tsteps) {
         fill_desc(c, c->plan_desc, c->plan);
-        fill_desc(c, c->plan1_desc, c->plan1);
+        if (c->plan1.tsteps) fill_desc(c, c->plan1_desc, c->plan1);
     }
     RD_CUDA(c, cudaMemcpyAsync(c->desc_dev, &c->desc, sizeof(InstDesc), cudaMemcpyHostToDevice,
                                c->stream));
@@ -889,6 +899,10 @@ rd_status step_ctx(rd_ctx* c, int64_t n) {
     const Use use = c->plan.tsteps == 0 || c->kernel != RD_KERNEL_MARCH ? Use::kTuning
                     : n >= c->plan.tsteps                               ? Use::kPlan
                                                                         : Use::kPlan1;
+    if (use == Use::kPlan1 && !c->plan1.tsteps) {   // first call of a single step
+        c->plan1 = default_plan(c->cfg, c->tun, 1);
+        fill_desc(c, c->plan1_desc, c->plan1);
+    }
     const rd_tuning& t = tuning_of(c, use);
     const int T = t.tsteps;
     int64_t full = n / T;
@@ -1017,7 +1031,7 @@ rd_status rd_create(const rd_config* cfg, rd_ctx** out) {
     c->own_stream = true;
     c->tun = default_tuning(c->cfg);
     c->plan = default_plan(c->cfg, c->tun, 2);
-    c->plan1 = default_plan(c->cfg, c->tun, 1);
+    if (c->plan.tsteps < 2) c->plan1 = c->plan;
     if (!(cfg->flags & RD_FLAG_NO_ALLOC)) {
         // owned from the first allocation on, so rd_destroy frees whatever
         // was obtained when a later one fails

@@ -229,8 +229,34 @@ struct XSides {
             xp[e] = (e < kVEC - 1) ? c[e + 1] : right;
         }
     }
+    // the same for a vector and those in the rows above and below (u, d):
+    // every shuffle first, then the predicated loads, which overwrite shuffled
+    // values and would stall the next row's shuffle
+    template <class ST, int ROWB>
+    __device__ __forceinline__ void get3(const float (&c)[kVEC], const float (&u)[kVEC],
+                                         const float (&d)[kVEC], const unsigned char* p,
+                                         float (&l)[3], float (&r)[3]) const {
+        constexpr unsigned FULL = 0xffffffffu;
+        l[0] = __shfl_up_sync(FULL, c[kVEC - 1], 1);
+        l[1] = __shfl_up_sync(FULL, u[kVEC - 1], 1);
+        l[2] = __shfl_up_sync(FULL, d[kVEC - 1], 1);
+        r[0] = __shfl_down_sync(FULL, c[0], 1);
+        r[1] = __shfl_down_sync(FULL, u[0], 1);
+        r[2] = __shfl_down_sync(FULL, d[0], 1);
+        const unsigned char* const pl = p + lcell * (int)sizeof(ST);
+        const unsigned char* const pr = p + rcell * (int)sizeof(ST);
+        lds_sides_if<ST>(l[0], r[0], pl, pr, llds, rlds);
+        lds_sides_if<ST>(l[1], r[1], pl - ROWB, pr - ROWB, llds, rlds);
+        lds_sides_if<ST>(l[2], r[2], pl + ROWB, pr + ROWB, llds, rlds);
+    }
     // the ghost beside a zero-flux face inside the vector, set to the face
     // cell in a thread's own copy of the vectors of one plane
+    __device__ __forceinline__ void set_ghost1(float (&c)[kVEC]) const {
+        if (!any_cut) return;
+        asm volatile("");   // keep the branch: rarely taken, uniform
+#pragma unroll
+        for (int e = kVEC - 1; e > 0; --e) c[e] = e == cut ? c[e - 1] : c[e];
+    }
     template <int S> __device__ __forceinline__ void set_ghost(float (&c)[S][kVEC]) const {
         if (!any_cut) return;
         asm volatile("");   // keep the branch: rarely taken, uniform
@@ -240,6 +266,12 @@ struct XSides {
             for (int e = kVEC - 1; e > 0; --e) c[s][e] = e == cut ? c[s][e - 1] : c[s][e];
     }
 };
+
+// A barrier of the whole CTA (nthreads: its size) for warps that run their own
+// loops: every warp passes it the same number of times, wherever in the code.
+__device__ __forceinline__ void cta_barrier(int nthreads) {
+    asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory");
+}
 
 // The global plane that the next copy reads, walked up from plane z0 - h:
 // wrapped (periodic z) or mirrored at zero-flux faces.

@@ -9,23 +9,25 @@
 
 namespace rdk {
 
-// Shared-memory ring of the 19-point kernel: planes q-1 .. q+4 rotate
-// through 6 slots; a slot holds, per species, (ty + 2) rows of kTileQ + 2
-// four-cell vectors and a four-cell guard at both ends.  96 halo fetch
-// descriptors follow the ring.
-constexpr int kRing19 = 6;
-__host__ __device__ inline int plane_elems19(int ty) {
-    return (ty + 2) * (kTileQ + 2) * 4 + 2 * 4;
+// Shared-memory ring of the 19-point kernel: planes q .. q+4 rotate through
+// 5 slots; a slot holds (ty + 2) rows of kTileQ + 2 four-cell vectors of
+// every field side by side (``mu_field``: one float field after the state's),
+// and a guard vector at both ends.
+constexpr int kRing19 = 5;
+constexpr int kGuard19 = 16;
+__host__ __device__ constexpr int row19_bytes(int nfields, int ebytes, bool mu_field) {
+    return (kTileQ + 2) * 4 * (nfields * ebytes + (mu_field ? 4 : 0));
 }
-__host__ __device__ inline size_t smem19_bytes(int nspecies, int ebytes, int ty) {
-    return (size_t)kRing19 * nspecies * plane_elems19(ty) * ebytes + 96 * 16;
+__host__ __device__ constexpr int plane19_bytes(int nfields, int ebytes, bool mu_field, int ty) {
+    return (ty + 2) * row19_bytes(nfields, ebytes, mu_field) + 2 * kGuard19;
 }
-// The same with ``mu_plane``: one more float plane per slot (the second
-// launch of a Cahn-Hilliard step, which reads mu beside the state).
-__host__ __device__ inline size_t smem19_pass_bytes(int nfields, int ebytes, bool mu_plane,
-                                                    int ty) {
-    return smem19_bytes(nfields, ebytes, ty) +
-           (mu_plane ? (size_t)kRing19 * plane_elems19(ty) * 4 : 0);
+__host__ __device__ constexpr size_t smem19_pass_bytes(int nfields, int ebytes, bool mu_field,
+                                                       int ty) {
+    // the ring, then 96 halo fetch descriptors
+    return (size_t)kRing19 * plane19_bytes(nfields, ebytes, mu_field, ty) + 96 * 16;
+}
+constexpr size_t smem19_bytes(int nspecies, int ebytes, int ty) {
+    return smem19_pass_bytes(nspecies, ebytes, false, ty);
 }
 inline int threads19(int ty) { return kTileQ * ty + 32; }
 

@@ -1,16 +1,16 @@
 // rd_step19_kernel.cuh -- one forward-Euler step of eq. (5) with the
-// 19-point Laplacian of eqs. (3)-(4), for the models without Cahn-Hilliard
-// (sm_103a).
+// 19-point Laplacian of eqs. (3)-(4) (sm_103a).
 //
-// Work items are those of the 7-point kernels: one thread per 4-cell vector of a 64 x TY tile plus one
-// halo warp, planes of the current state copied into a shared-memory ring
-// by per-thread cp.async several planes ahead, one barrier per plane.  What
-// differs:
+// Work items, copies, thread layout and boundary rules are those of
+// rd_march_kernel at one step per launch: one thread per 4-cell vector of a
+// 64 x TY tile plus one halo warp, planes of the current state copied into a
+// shared-memory ring by 16-byte cp.async several planes ahead, rows holding
+// every field side by side, one barrier per plane, register sets that change
+// roles from plane to plane, x neighbours by warp shuffle.  What differs:
 //
 //  * Neighbourhood.  A cell reads the 3x3 block of its own plane (weights
 //    -24 centre, 2 faces, 1 diagonals) and the 5-point cross of the planes
-//    below and above (2 centre, 1 faces); corners weigh 0.  The diagonals
-//    need the tile's four corner vectors, which the halo warp also copies.
+//    below and above (2 centre, 1 faces); corners weigh 0.
 //  * Per-plane sums carried down the march.  When plane k arrives, a
 //    thread forms at each of its 4 cells, with X = xm + xp + ym + yp,
 //        Z_k = 2 c + X                 (plane k as a z-neighbour)
@@ -18,20 +18,22 @@
 //    so that 6 h^2 Lap c on plane q = W_q - 24 c_q + Z_{q-1} + Z_{q+1}.
 //    Z_{q-1}, Z_q, W_q and c_q stay in registers; each plane is read from
 //    shared memory once, on arrival (plane q+1 at step q).
-//  * Ring reuse.  A plane's last reads are its arrival and, with wind, the
-//    two elements beside a thread's own row at its own step, so the copy
-//    issued at step q may overwrite plane q-2, whose reads all ended before
-//    the barrier of step q-1: the 7-point kernel's ring of 6 slots with
-//    P = 5 copy groups ahead of q-1.  The first step of a work item also
-//    reads the neighbours of plane z0-1, whose slot the copy of step z0+1
-//    refills; one more barrier after those reads keeps the rule.
+//  * Ring reuse.  At step q the slot of plane q-1 is refilled; its
+//    neighbours were read at step q-2 (on arrival) and, with wind, q-1; the
+//    sums of a work item's first two planes are formed before its first step.
 //
-// Boundary rules are those of the 7-point kernels: ghost rows, planes and
-// vectors are copied in under each axis's rule (zero flux: the face value;
-// periodic: wrapped), and a thread at a zero-flux x face reads the cells
-// beyond it from its own column (xface_offsets), so an edge ghost composes
-// the rules of the two axes it crosses, as the paper fills its edges after
-// its faces (Section 4.1); a held layer's cell takes its bc value.
+// Measured against the kernel before it (scalar arithmetic, single-element
+// shared loads with a 4-way bank conflict, sums of the field rows moved from
+// register to register), best tilings: 192^3 Turing 248 -> 316 GLUPS, the
+// 192^3 Cahn-Hilliard step 84 -> 112, the 144 x 144 x 384 plume 194 -> 247.
+// It is bound by latency: 12 to 18 warps on an SM wait on one another's
+// barrier and on shuffles and shared loads.
+//
+// An edge ghost composes the rules of the two axes it crosses, as the paper
+// fills its edges after its faces (Section 4.1): rows beyond a zero-flux y
+// face are copied in as the face row, and a thread at a zero-flux x face
+// reads its own column in the rows above and below too.  A held layer's cell
+// takes its bc value.
 #pragma once
 
 #include "rd_step19.h"
@@ -49,50 +51,57 @@ namespace rdk {
 // to c.  The ring of PASS 1 holds species 2 only.
 template <class M, class ST, int PASS> struct Layout19 {
     static constexpr int S = M::S;
-    static constexpr int NS = PASS == 1 ? 1 : S;    // state fields per slot
-    static constexpr bool MUF = PASS == 2;          // plus one float mu plane
+    static constexpr int NS = PASS == 1 ? 1 : S;    // state fields per row
+    static constexpr bool MUF = PASS == 2;          // plus one float mu field
     static constexpr int RING = kRing19;
-    static constexpr int P = 5;
-    static_assert(RING == P + 1, "the copy of step q refills the slot of plane q - 2");
+    static constexpr int P = RING;                  // planes issued ahead of q - 1
+    static constexpr int SPB = kRW * (int)sizeof(ST);
+    static constexpr int ROWB = row19_bytes(NS, (int)sizeof(ST), MUF);
+    static_assert(ROWB % 16 == 0 && (NS * SPB) % 16 == 0, "16-byte vectors");
     static_assert(PASS == 0 || M::CH, "passes 1 and 2 are for Cahn-Hilliard models");
-    __host__ __device__ static int plane_elems(int ty) { return plane_elems19(ty); }
+    // registers a thread may take (measured best tilings, GLUPS): the
+    // one-species plume 250 (80) 239 (96) 231 (128); two-species Turing 192^3
+    // 275 (80) 311 (96) 319 (128); the Cahn-Hilliard step 72 (80) 102 (128)
+    static constexpr int regs() {
+        return NS == 1 && PASS == 0 && sizeof(ST) == 4 ? 80 : 128;
+    }
+    __host__ __device__ static int plane_bytes(int ty) {
+        return plane19_bytes(NS, (int)sizeof(ST), MUF, ty);
+    }
     __host__ __device__ static size_t total(int ty) {
         return smem19_pass_bytes(NS, (int)sizeof(ST), MUF, ty);
     }
     __host__ __device__ static int threads(int ty) { return kTileQ * ty + 32; }
 };
 
-// Own vector c and the sums Z, W of one species plane at the thread's 4
-// cells; ``p`` points at the own vector in the ring, ``loff`` / ``roff``
-// are the byte offsets of the x neighbours beside it (xface_offsets: at a
-// zero-flux x face, the thread's own face cell, also in the rows above and
-// below, where the edge ghost composes both faces' rules).
-template <class ST>
-__device__ __forceinline__ void plane_sums19(const unsigned char* p, int loff, int roff,
+// Own vector c and the sums Z, W of one field's plane at the thread's 4
+// cells; ``p`` points at the own vector in the ring, rows ROWB bytes apart.
+// The x neighbours of a pair are no aligned pair of registers: sums along x
+// are taken cell by cell, everything else packed.
+template <class ST, int ROWB>
+__device__ __forceinline__ void plane_sums19(const XSides& sides, const unsigned char* p,
                                              float (&c)[kVEC], float (&zs)[kVEC],
                                              float (&ws)[kVEC]) {
-    constexpr int RWB = kRW * (int)sizeof(ST);
-    float ym[kVEC], yp[kVEC];
+    float ym[kVEC], yp[kVEC], l[3], r[3];
     lds_vec<ST>(p, c);
-    lds_vec<ST>(p - RWB, ym);
-    lds_vec<ST>(p + RWB, yp);
-    const unsigned char* pl = p + loff;
-    const unsigned char* pr = p + roff;
-    const float l = lds_one<ST>(pl), r = lds_one<ST>(pr);
-    const float ul = lds_one<ST>(pl - RWB), ur = lds_one<ST>(pr - RWB);
-    const float dl = lds_one<ST>(pl + RWB), dr = lds_one<ST>(pr + RWB);
+    lds_vec<ST>(p - ROWB, ym);
+    lds_vec<ST>(p + ROWB, yp);
+    sides.set_ghost1(c);
+    sides.set_ghost1(ym);
+    sides.set_ghost1(yp);
+    sides.get3<ST, ROWB>(c, ym, yp, p, l, r);
+    // xm + xp of the pair h of a row with the elements le, re beside it
+    auto xpair = [](const float(&v)[kVEC], float le, float re, int h) {
+        return h ? make_float2(__fadd_rn(v[1], v[3]), __fadd_rn(v[2], re))
+                 : make_float2(__fadd_rn(le, v[1]), __fadd_rn(v[0], v[2]));
+    };
 #pragma unroll
-    for (int e = 0; e < kVEC; ++e) {
-        const float xm = e ? c[e - 1] : l;
-        const float xp = e < kVEC - 1 ? c[e + 1] : r;
-        const float yml = e ? ym[e - 1] : ul;
-        const float ymr = e < kVEC - 1 ? ym[e + 1] : ur;
-        const float ypl = e ? yp[e - 1] : dl;
-        const float ypr = e < kVEC - 1 ? yp[e + 1] : dr;
-        const float cross = __fadd_rn(__fadd_rn(xm, xp), __fadd_rn(ym[e], yp[e]));
-        const float diag = __fadd_rn(__fadd_rn(yml, ymr), __fadd_rn(ypl, ypr));
-        zs[e] = __fmaf_rn(2.0f, c[e], cross);
-        ws[e] = __fmaf_rn(2.0f, cross, diag);
+    for (int h = 0; h < 2; ++h) {
+        const float2 cross =
+            vadd(xpair(c, l[0], r[0], h), vadd(pair_of(ym, h), pair_of(yp, h)));
+        const float2 diag = vadd(xpair(ym, l[1], r[1], h), xpair(yp, l[2], r[2], h));
+        set_pair(zs, h, vfma(vset<float2>(2.0f), pair_of(c, h), cross));
+        set_pair(ws, h, vfma(vset<float2>(2.0f), cross, diag));
     }
 }
 
@@ -131,35 +140,16 @@ __device__ __forceinline__ void species19(const InstDesc& sd, int s, float k6,
         }
     }
 #pragma unroll
-    for (int e = 0; e < kVEC; ++e) o[e] = __fadd_rn(c[e], __fmaf_rn(k6, lap6[e], in[e]));
-}
-
-// One float field of a plane (the mu plane of PASS 2), fetched with the
-// state's descriptor: the same rows, pitch and ghost rules.  ``mu0`` is the
-// address of the mu plane's element 0.
-template <class ST>
-__device__ __forceinline__ void fetch_mu(const Fetch& f, unsigned char* mu0,
-                                         const float* gplane, int nx, bool elems, bool px,
-                                         const InstDesc& sd) {
-    float* d = reinterpret_cast<float*>(mu0 + f.soff / (int)sizeof(ST) * 4);
-    const int ok = f.mode == 1 && RD_DBG_GLOBAL(sd, gplane + f.goff, 16, kSiteMu);
-    Store<float>::cp_async_if(d, gplane + f.goff, ok);
-    if (elems && f.mode == 2) {
-#pragma unroll
-        for (int e = 0; e < kVEC; ++e) {
-            const int x = f.xs + e;
-            const int xi = px ? wrapi(x, nx) : (x < 0 ? 0 : (x >= nx ? nx - 1 : x));
-            if (RD_DBG_GLOBAL(sd, gplane + f.goff + xi, 4, kSiteMu))
-                Store<float>::cp_async_elem(d + e, gplane + f.goff + xi);
-        }
-    }
+    for (int h = 0; h < 2; ++h)
+        set_pair(o, h, vadd(pair_of(c, h),
+                            vfma(vset<float2>(k6), pair_of(lap6, h), pair_of(in, h))));
 }
 
 // PLAIN: no held layer, point source or wind.  PASS: see Layout19.  W3:
 // the 3-D wind (upwind along y and z too; never with PLAIN, PASS 0 only).
 template <class M, class ST, bool ONE, bool PLAIN, int PASS, bool W3 = false>
-__global__ void __launch_bounds__(kMaxThreads, 1)
-rd_step19_kernel(const __grid_constant__ LaunchArgs a) {
+__global__ void __maxnreg__((Layout19<M, ST, PASS>::regs()))
+rd_march19_kernel(const __grid_constant__ LaunchArgs a) {
     using LY = Layout19<M, ST, PASS>;
     constexpr int S = M::S;
     constexpr int NS = LY::NS;
@@ -170,6 +160,9 @@ rd_step19_kernel(const __grid_constant__ LaunchArgs a) {
     constexpr int P = LY::P;
     constexpr int RING = LY::RING;
     constexpr int EB = (int)sizeof(ST);
+    constexpr int SPB = LY::SPB;
+    constexpr int ROWB = LY::ROWB;
+    constexpr unsigned FULL = 0xffffffffu;
 
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ InstDesc sdm;
@@ -178,21 +171,16 @@ rd_step19_kernel(const __grid_constant__ LaunchArgs a) {
 
     const int tid = threadIdx.x;
     const int TY = a.ty;
-    const int PE = LY::plane_elems(TY);
-    const int PEB = PE * EB;                                 // bytes per state plane
-    const int SLOTB = NS * PEB + (MUF ? PE * 4 : 0);         // bytes per ring slot
-    unsigned char* const ring = smem + kVEC * EB;            // slot 0, field 0
+    const int SLOTB = LY::plane_bytes(TY);
+    const int ninner = kTileQ * TY;
+    const TilePos t(min(tid, ninner + TilePos::ring(TY) - 1), TY);
+    const int hl = tid - ninner;                             // >= 0: halo thread
+    const bool inner = hl < 0;
+    const bool inner_warp = __all_sync(FULL, inner);         // TY is even
+    // byte offsets of the own vector, in the state fields and in mu, slot 0
+    const int own0 = kGuard19 + t.r * ROWB + t.v * kVEC * EB;
     int4* const hfetch = reinterpret_cast<int4*>(smem + RING * SLOTB);
-    const int ncomp = kTileQ * TY;
-    const bool halo_warp = tid >= ncomp;
-    const int r = tid / kTileQ;
-    const int v = tid - r * kTileQ;
-    const int own_e = (r + 1) * kRW + (v + 1) * kVEC;        // element offset in a plane
-    const int own_b = own_e * EB;
-    // the mu plane of a slot (PASS 2) starts at NS * PEB; its guard is
-    // kVEC floats, the state planes' kVEC elements of ST
-    const int mu0_b = NS * PEB + kVEC * (4 - EB);            // element 0, from a slot
-    const int mu_own_b = mu0_b + own_e * 4;
+    const int mu_own = NS * SPB + t.v * kVEC * (4 - EB);     // from the own vector
 
     int cur_inst = -1;
     if (tid == 0) s_inst = 0;
@@ -204,7 +192,6 @@ rd_step19_kernel(const __grid_constant__ LaunchArgs a) {
 
         const int nx = sd.nx, ny = sd.ny, nz = sd.nz, pitch = sd.pitch;
         const bool px = sd.per_x, py = sd.per_y, pz = sd.per_z;
-        const bool elems = sd.wrap_elems || !sd.per_x;
         const long long local = item - sd.item_begin;
         const int txi = (int)(local % sd.ntx);
         const int tyi = (int)((local / sd.ntx) % sd.nty);
@@ -216,55 +203,18 @@ rd_step19_kernel(const __grid_constant__ LaunchArgs a) {
         const ST* const gin = reinterpret_cast<const ST*>(sd.base[lin][PASS == 1 ? 2 : 0]);
         ST* const gout = reinterpret_cast<ST*>(sd.base[lin ^ 1][0]);
         const long long fstride =
-            NS > 1 ? reinterpret_cast<const ST*>(sd.base[lin][1]) - gin : 0;
+            S > 1 ? reinterpret_cast<const ST*>(sd.base[lin][1]) -
+                        reinterpret_cast<const ST*>(sd.base[lin][0])
+                  : 0;
         const long long plane = sd.plane;
 
-        // ---- halo lanes: 2 TY side vectors, 2 x 16 row vectors, then the 4
-        // corner vectors (rows -1 and TY, vector columns -1 and 16)
-        if (halo_warp) {
-            const int hl = tid - ncomp;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const int j = hl + 32 * k;
-                Fetch f{0, 0, 0, 0};
-                if (j < 2 * TY) {
-                    const int hr = j >> 1;
-                    const bool right = j & 1;
-                    const int xh = right ? x0 + kTileQ * kVEC : x0 - kVEC;
-                    f = make_fetch<ST>(y0 + hr, xh, nx, ny, pitch, px, py,
-                                       (hr + 1) * kRW + (right ? kNQ - 1 : 0) * kVEC, true);
-                } else if (j < 2 * TY + 2 * kTileQ) {
-                    const int jj = j - 2 * TY;
-                    const bool bottom = jj >= kTileQ;
-                    const int hv = jj - (bottom ? kTileQ : 0);
-                    f = make_fetch<ST>(bottom ? y0 + TY : y0 - 1, x0 + hv * kVEC, nx, ny, pitch, px,
-                                       py, (bottom ? TY + 1 : 0) * kRW + (hv + 1) * kVEC, true);
-                } else if (j < 2 * TY + 2 * kTileQ + 4) {
-                    const int jj = j - 2 * TY - 2 * kTileQ;
-                    const bool bottom = jj >= 2;
-                    const bool right = jj & 1;
-                    f = make_fetch<ST>(bottom ? y0 + TY : y0 - 1,
-                                       right ? x0 + kTileQ * kVEC : x0 - kVEC, nx, ny, pitch, px,
-                                       py,
-                                       (bottom ? TY + 1 : 0) * kRW + (right ? kNQ - 1 : 0) * kVEC,
-                                       true);
-                }
-                if (RD_DBG_SHARED(hfetch + j, 16, kSiteHaloDesc))
-                    hfetch[j] = make_int4(f.mode, f.goff, f.soff, f.xs);
-            }
-        }
-        // ---- compute threads: own vector
-        const int y = y0 + r;
-        const int xs = x0 + v * kVEC;
-        const bool computes = !halo_warp && y < ny && xs < nx;
-        const bool src_col = sd.src_s >= 0 && (py ? wrapi(y, ny) : y) == sd.src_y;
+        const int y = y0 - 1 + t.r;                   // global row of the position
+        const int xs = x0 - kVEC + t.v * kVEC;        // global x of its first element
+        const bool stores = inner && y < ny && xs < nx;
+        const XSides sides(t, inner, xs, x0, nx, px);
         const unsigned xyf = xy_faces(xs, y, nx, ny);
-        const Fetch fo = halo_warp ? Fetch{0, 0, 0, 0}
-                                   : make_fetch<ST>(y, xs, nx, ny, pitch, px, py, own_e, true);
-        int loff, roff;                           // x neighbours beside the own vector
-        xface_offsets<ST>(xs, nx, px, loff, roff);
-        int loff_f = 0, roff_f = 0;               // the same in the float mu plane
-        if constexpr (MUF) xface_offsets<float>(xs, nx, px, loff_f, roff_f);
+        const bool src_col = sd.src_s >= 0 && (py ? wrapi(y, ny) : y) == sd.src_y;
+        const bool elems = sd.wrap_elems;
         // k6: D dt / (6 h^2) per species; PASS 1: p[2] / 6 (mu); PASS 2:
         // k6[2] = p[1] / 6 (the mobility term of c)
         float k6[S];
@@ -272,108 +222,145 @@ rd_step19_kernel(const __grid_constant__ LaunchArgs a) {
         for (int s = 0; s < S; ++s) k6[s] = __fdiv_rn(sd.kx[s], 6.0f);
         if constexpr (PASS == 1) k6[0] = __fdiv_rn(sd.p[2], 6.0f);
         if constexpr (PASS == 2) k6[2] = __fdiv_rn(sd.p[1], 6.0f);
-        float cy = 0.0f, cz = 0.0f;               // 3-D wind
+        float cy = 0.0f, cz = 0.0f;                   // 3-D wind
         if constexpr (W3 && PASS == 0) wind3d(sd, lin, local, cy, cz);
-        __syncthreads();   // halo descriptors written
+        // what the thread copies of every plane: its own vector, element
+        // offset ``go`` of a plane (-1: none, -2: element by element), or for
+        // the halo warp three vectors a lane, described in shared memory
+        int go = -1;
+        if (inner) {
+            const Fetch f = make_fetch_h<ST>(y, xs, nx, ny, pitch, px, py, 0);
+            go = f.mode == 1 ? f.goff : -f.mode;
+        } else {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const int j = min(tid + 32 * k, ninner + TilePos::ring(TY) - 1);
+                const TilePos h(j, TY);
+                const Fetch f = make_fetch_h<ST>(y0 - 1 + h.r, x0 - kVEC + h.v * kVEC, nx, ny,
+                                                 pitch, px, py,
+                                                 kGuard19 + h.r * ROWB + h.v * kVEC * EB);
+                if (RD_DBG_SHARED(hfetch + hl + 32 * k, 16, kSiteHaloDesc))
+                    hfetch[hl + 32 * k] = make_int4(f.mode, f.goff, f.soff, f.xs);
+            }
+            __syncwarp();
+        }
+        // from a vector's place in the state fields to that in mu
+        auto mu_shift = [&](int vx) { return NS * SPB + ((vx - x0) + kVEC) * (4 - EB); };
 
-        // ---- the march: plane nld is fetched P planes ahead into slot sl;
-        // plane z0 - 1 goes to slot 0, plane q to slot (q - z0 + 1) mod RING
-        int nld = z0 - 1;
-        int zld = pz ? wrapi(nld, nz) : nld;
-        auto issue = [&](int sl) {
-            const bool in_z = pz || (nld >= 0 && nld < nz);
-            if (nld <= z1) {
-                const int zs = in_z ? zld : (nld < 0 ? 0 : nz - 1);
-                const ST* gld = gin + (long long)zs * plane;
-                const float* gmu = nullptr;
-                if constexpr (MUF) gmu = sd.mu + (long long)zs * plane;
-                unsigned char* buf = ring + sl * SLOTB;
-                if (halo_warp) {
-                    const int hl = tid - ncomp;
+        // planes z0-1 .. z1 are copied; the next one to slot_ld
+        PlaneFeed feed(z0 - 1, nz, pz);
+        const int slot_end = own0 + RING * SLOTB;
+        int slot_ld = own0;
+        // the vector at element offset o of the plane at goff, to d (mu: dm)
+        auto copy = [&](long long goff, int o, unsigned char* d, unsigned char* dm, bool ok) {
+            const ST* const g = gin + goff + o;
+#pragma unroll
+            for (int s = 0; s < NS; ++s)
+                Store<ST>::cp_async_if(
+                    reinterpret_cast<ST*>(d + s * SPB), g + s * fstride,
+                    ok && RD_DBG_GLOBAL(sd, g + s * fstride, 4 * (int)sizeof(ST), kSiteCopySrc));
+            if constexpr (MUF) {
+                const float* const gm = sd.mu + goff + o;
+                Store<float>::cp_async_if(reinterpret_cast<float*>(dm), gm,
+                                          ok && RD_DBG_GLOBAL(sd, gm, 16, kSiteMu));
+            }
+        };
+        auto copy_elems = [&](long long goff, Fetch f, unsigned char* d) {
+            fetch_elems<ST, NS>(f, d, SPB, gin + goff, fstride, nx, sd);
+            if constexpr (MUF) {
+                f.soff += mu_shift(f.xs);
+                fetch_elems<float, 1>(f, d, 0, sd.mu + goff, 0, nx, sd);
+            }
+        };
+        auto issue = [&]() {
+            if (feed.n <= z1) {
+                const long long goff = (long long)feed.plane() * plane;
+                unsigned char* const d = smem + slot_ld;
+                if (inner_warp) {
+                    copy(goff, go, d, d + mu_own, go >= 0);
+                } else {
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
-                        int4 h = make_int4(0, 0, 0, 0);
-                        if (RD_DBG_SHARED(hfetch + hl + 32 * k, 16, kSiteHaloDesc))
-                            h = hfetch[hl + 32 * k];
-                        const Fetch f{h.x, h.y, h.z, h.w};
-                        fetch_all<ST, NS>(f, buf, PEB, gld, fstride, nx, elems, px, sd);
-                        if constexpr (MUF) fetch_mu<ST>(f, buf + mu0_b, gmu, nx, elems, px, sd);
+                        const int4 h = hfetch[hl + 32 * k];
+                        unsigned char* const dk = d - own0 + h.z;
+                        copy(goff, h.y, dk, dk + mu_shift(h.w), h.x == 1);
                     }
-                } else {
-                    fetch_all<ST, NS>(fo, buf, PEB, gld, fstride, nx, elems, px, sd);
-                    if constexpr (MUF) fetch_mu<ST>(fo, buf + mu0_b, gmu, nx, elems, px, sd);
+                }
+                if (elems) {   // periodic x, nx not a multiple of 4
+                    if (go == -2)
+                        copy_elems(goff, make_fetch_h<ST>(y, xs, nx, ny, pitch, px, py, 0), d);
+                    if (!inner_warp)
+                        for (int k = 0; k < 3; ++k) {
+                            const int4 h = hfetch[hl + 32 * k];
+                            copy_elems(goff, Fetch{h.x, h.y, h.z, h.w}, d - own0);
+                        }
                 }
             }
-            ++nld;
-            if (!pz) zld = nld;
-            else if (++zld == nz) zld = 0;
+            feed.next();
+            slot_ld += SLOTB;
+            if (slot_ld == slot_end) slot_ld = own0;
             cp_async_commit();
         };
-        // plane sums of field f of the slot at ``base`` (own vector address)
-        auto sums = [&](const unsigned char* base, int f, float (&c)[kVEC], float (&zs)[kVEC],
-                        float (&ws)[kVEC]) {
-            if (MUF && f == NSUM - 1)
-                plane_sums19<float>(base - own_b + mu_own_b, loff_f, roff_f, c, zs, ws);
-            else
-                plane_sums19<ST>(base + f * PEB, loff, roff, c, zs, ws);
+        // plane sums of field i of the slot whose own vector is at ``p``
+        auto sums = [&](const unsigned char* p, int i, float(&c)[kVEC], float(&zs)[kVEC],
+                        float(&ws)[kVEC]) {
+            if (MUF && i == NSUM - 1) plane_sums19<float, ROWB>(sides, p + mu_own, c, zs, ws);
+            else plane_sums19<ST, ROWB>(sides, p + i * SPB, c, zs, ws);
         };
 #pragma unroll 1
-        for (int j = 0; j < P; ++j) issue(j);
-        int zq = pz ? wrapi(z0, nz) : z0;
+        for (int j = 0; j < P; ++j) issue();
+
         ST* gst = gout + (long long)z0 * plane + (long long)y * pitch + xs;
         float* gmu_st = nullptr;
         if constexpr (PASS == 1) gmu_st = sd.mu + (long long)z0 * plane + (long long)y * pitch + xs;
-        const float* courant = sd.courant;
-        int sc = 1;                               // ring slot of plane q
-        // sums of planes q-1 and q, and the own vector of plane q
-        float zsum_m[NSUM][kVEC], zsum_0[NSUM][kVEC], wsum_0[NSUM][kVEC], c_0[NSUM][kVEC];
-        float cc_0[kVEC];                         // PASS 2: own c of plane q
-#pragma unroll 1
-        for (int q = z0; q < z1; ++q) {
-            const int sm = sc == 0 ? RING - 1 : sc - 1;
-            const int sp = sc == RING - 1 ? 0 : sc + 1;
-            // overwrite plane q - 2; planes up to q + 1 must have landed
-            issue(sc + P - 1 >= RING ? sc + P - 1 - RING : sc + P - 1);
-            cp_async_wait<P - 2>();
-            __syncthreads();
-            const unsigned char* Pc = ring + sc * SLOTB + own_b;
-            if (q == z0) {   // block-uniform
-                if (!halo_warp) {
-                    const unsigned char* Pm = ring + sm * SLOTB + own_b;
+        int slot = own0;                              // ring slot of plane q - 1
+        auto next_slot = [&](int x) {
+            x += SLOTB;
+            return x == slot_end ? own0 : x;
+        };
+        // three sets each of the sums and own vectors, roles rotating; CC: the
+        // own c of PASS 2
+        float ZA[NSUM][kVEC], ZB[NSUM][kVEC], ZC[NSUM][kVEC];
+        float WA[NSUM][kVEC], WB[NSUM][kVEC], WC[NSUM][kVEC];
+        float CA[NSUM][kVEC], CB[NSUM][kVEC], CC[NSUM][kVEC];
+        float DA[kVEC], DB[kVEC], DC[kVEC];
+        // the step for plane q: sums of planes q - 1 and q in zm and z0, w0,
+        // own vectors of planes q - 1 and q in cm and c0; those of plane
+        // q + 1 are formed here
+        auto body = [&](int q, float(&zm)[NSUM][kVEC], float(&zq)[NSUM][kVEC],
+                        float(&zp)[NSUM][kVEC], float(&wq)[NSUM][kVEC], float(&wp)[NSUM][kVEC],
+                        float(&cm)[NSUM][kVEC], float(&c0)[NSUM][kVEC], float(&cp)[NSUM][kVEC],
+                        float(&dq)[kVEC], float(&dp)[kVEC]) {
+            // planes through q + 1 must have landed: of those issued, through
+            // q + P - 2, all but the newest P - 3
+            cp_async_wait<P - 3>();
+            cta_barrier(blockDim.x);
+            const int s0 = next_slot(slot);
+            const unsigned char* const p0 = smem + s0;
+            {
+                const unsigned char* const p1 = smem + next_slot(s0);
+                if constexpr (PASS == 2) lds_vec<ST>(p1 + 2 * SPB, dp);
+                float lap6[NSUM][kVEC];   // 6 h^2 Lap of the fields on plane q
 #pragma unroll
-                    for (int f = 0; f < NSUM; ++f) {
-                        float cm[kVEC], wm[kVEC];
-                        sums(Pm, f, cm, zsum_m[f], wm);
-                        sums(Pc, f, c_0[f], zsum_0[f], wsum_0[f]);
-                    }
-                    if constexpr (PASS == 2) lds_vec<ST>(Pc + 2 * PEB, cc_0);
+                for (int i = 0; i < NSUM; ++i) {
+                    sums(p1, i, cp[i], zp[i], wp[i]);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        set_pair(lap6[i], h,
+                                 vfma(vset<float2>(-24.0f), pair_of(c0[i], h),
+                                      vadd(vadd(pair_of(zm[i], h), pair_of(zp[i], h)),
+                                           pair_of(wq[i], h))));
                 }
-                __syncthreads();   // plane z0 - 1 is refilled at the next step
-            }
-            if (!halo_warp) {
-                const unsigned char* Pp = ring + sp * SLOTB + own_b;
-                float c_p[NSUM][kVEC], zsum_p[NSUM][kVEC], wsum_p[NSUM][kVEC];
-                float cc_p[kVEC];
-#pragma unroll
-                for (int f = 0; f < NSUM; ++f) sums(Pp, f, c_p[f], zsum_p[f], wsum_p[f]);
-                if constexpr (PASS == 2) lds_vec<ST>(Pp + 2 * PEB, cc_p);
-                // 6 h^2 Lap of each summed field on plane q
-                float lap6[NSUM][kVEC];
-#pragma unroll
-                for (int f = 0; f < NSUM; ++f)
-#pragma unroll
-                    for (int e = 0; e < kVEC; ++e)
-                        lap6[f][e] = __fmaf_rn(-24.0f, c_0[f][e],
-                                               __fadd_rn(__fadd_rn(zsum_m[f][e], zsum_p[f][e]),
-                                                         wsum_0[f][e]));
                 if constexpr (PASS == 1) {
                     // mu = g(c) - (p[2] / 6) 6 h^2 Lap c
                     float mu[kVEC];
 #pragma unroll
-                    for (int e = 0; e < kVEC; ++e)
-                        mu[e] = __fmaf_rn(-k6[0], lap6[0][e], M::g(sd, c_0[0][e]));
-                    if (computes && RD_DBG_GLOBAL(sd, gmu_st, 16, kSiteMu))
+                    for (int h = 0; h < 2; ++h)
+                        set_pair(mu, h, vfma(vset<float2>(-k6[0]), pair_of(lap6[0], h),
+                                             M::g(sd, pair_of(c0[0], h))));
+                    if (stores && RD_DBG_GLOBAL(sd, gmu_st, 16, kSiteMu))
                         Store<float>::store(gmu_st, mu);
+                    gmu_st += plane;
                 } else {
                     // state of plane q: a, b (and every PASS 0 species) from
                     // the summed fields, c of PASS 2 from its own vector
@@ -381,34 +368,24 @@ rd_step19_kernel(const __grid_constant__ LaunchArgs a) {
 #pragma unroll
                     for (int s = 0; s < S; ++s)
 #pragma unroll
-                        for (int e = 0; e < kVEC; ++e)
-                            cen[s][e] = (PASS == 2 && s == 2) ? cc_0[e] : c_0[s][e];
-#pragma unroll
-                    for (int e = 0; e < kVEC; ++e) {
-                        float cv[S], iv[S];
-#pragma unroll
-                        for (int s = 0; s < S; ++s) cv[s] = cen[s][e];
-                        M::react(sd, cv, iv);
-#pragma unroll
-                        for (int s = 0; s < S; ++s) inc[s][e] = iv[s];
-                    }
+                        for (int i = 0; i < kVEC; ++i)
+                            cen[s][i] = (PASS == 2 && s == 2) ? dq[i] : c0[s < NSUM ? s : 0][i];
+                    react4<M>(sd, cen, inc);
                     if (W3 && (cy != 0.0f || cz != 0.0f)) {
-                        // upwind along y and z (3-D wind): y neighbours from
-                        // plane q, z neighbours from the thread's own column
-                        // in planes q - 1 (still in the ring) and q + 1
-                        const unsigned char* Pm = ring + sm * SLOTB + own_b;
+                        // upwind along y and z (3-D wind): y neighbours of
+                        // plane q, z neighbours the thread's own vectors
 #pragma unroll
                         for (int s = 0; s < S; ++s) {
-                            float ym[kVEC], yp[kVEC], zm[kVEC];
-                            lds_vec<ST>(Pc + s * PEB - kRW * EB, ym);
-                            lds_vec<ST>(Pc + s * PEB + kRW * EB, yp);
-                            lds_vec<ST>(Pm + s * PEB, zm);
+                            float ym[kVEC], yp[kVEC];
+                            lds_vec<ST>(p0 + s * SPB - ROWB, ym);
+                            lds_vec<ST>(p0 + s * SPB + ROWB, yp);
                             upwind_axis(cy, cen[s], ym, yp, inc[s]);
-                            upwind_axis(cz, cen[s], zm, c_p[s < NSUM ? s : 0], inc[s]);
+                            upwind_axis(cz, cen[s], cm[s < NSUM ? s : 0], cp[s < NSUM ? s : 0],
+                                        inc[s]);
                         }
                     }
-                    const float cx = PLAIN ? 0.0f : courant_at(sd, courant, zq);
-                    const bool src_here = src_col && zq == sd.src_z;
+                    const float cx = PLAIN ? 0.0f : courant_at(sd, sd.courant, q);
+                    const bool src_here = src_col && q == sd.src_z;
                     const unsigned faces = xyf | z_faces(q, nz);
 #pragma unroll
                     for (int s = 0; s < S; ++s) {
@@ -417,35 +394,52 @@ rd_step19_kernel(const __grid_constant__ LaunchArgs a) {
                         const float(&ls)[kVEC] = lap6[(PASS == 2 && s == 2) ? 2 : (s < NSUM ? s : 0)];
                         float left = 0.0f, right = 0.0f;
                         if (!PLAIN && cx != 0.0f) {
-                            left = lds_one<ST>(Pc + s * PEB + loff);
-                            right = lds_one<ST>(Pc + s * PEB + roff);
+                            const unsigned char* ps = p0 + s * SPB;
+                            left = lds_one<ST>(ps + sides.lcell * EB);
+                            // (a face inside the vector: cen holds the ghost)
+                            right = lds_one<ST>(ps + sides.rcell * EB);
                         }
                         species19<PLAIN>(sd, s, k6[s], cen[s], ls, inc[s], cx, left, right,
                                          src_here, px, xs, o);
                         if constexpr (!PLAIN) held_layers_at(sd, s, faces, xs, y, q, o);
-                        if (computes && RD_DBG_GLOBAL(sd, gst + s * fstride, 4 * (int)sizeof(ST),
-                                                      kSiteStateStore))
+                        if (stores && RD_DBG_GLOBAL(sd, gst + s * fstride, 4 * (int)sizeof(ST),
+                                                    kSiteStateStore))
                             Store<ST>::store(gst + s * fstride, o);
                     }
+                    gst += plane;
                 }
-#pragma unroll
-                for (int f = 0; f < NSUM; ++f)
-#pragma unroll
-                    for (int e = 0; e < kVEC; ++e) {
-                        zsum_m[f][e] = zsum_0[f][e];
-                        zsum_0[f][e] = zsum_p[f][e];
-                        wsum_0[f][e] = wsum_p[f][e];
-                        c_0[f][e] = c_p[f][e];
-                    }
-                if constexpr (PASS == 2)
-#pragma unroll
-                    for (int e = 0; e < kVEC; ++e) cc_0[e] = cc_p[e];
             }
-            gst += plane;
-            if constexpr (PASS == 1) gmu_st += plane;
-            sc = sc == RING - 1 ? 0 : sc + 1;
-            if (!pz) zq = q + 1;
-            else if (++zq == nz) zq = 0;
+            // refills the slot of plane q - 1; last, behind the step's own loads
+            issue();
+            slot = s0;
+        };
+        // the sums of the first two planes, formed before the first barrier of
+        // the march, after which their slots are refilled
+        cp_async_wait<P - 2>();
+        cta_barrier(blockDim.x);
+        if (inner_warp) {
+            float w[kVEC];
+#pragma unroll
+            for (int i = 0; i < NSUM; ++i) {
+                sums(smem + slot, i, CA[i], ZA[i], w);
+                sums(smem + next_slot(slot), i, CB[i], ZB[i], WA[i]);
+            }
+            if constexpr (PASS == 2) lds_vec<ST>(smem + next_slot(slot) + 2 * SPB, DA);
+            for (int q = z0;;) {
+                body(q, ZA, ZB, ZC, WA, WB, CA, CB, CC, DA, DB);
+                if (++q == z1) break;
+                body(q, ZB, ZC, ZA, WB, WC, CB, CC, CA, DB, DC);
+                if (++q == z1) break;
+                body(q, ZC, ZA, ZB, WC, WA, CC, CA, CB, DC, DA);
+                if (++q == z1) break;
+            }
+        } else {   // the halo warp only copies
+#pragma unroll 1
+            for (int q = z0; q < z1; ++q) {
+                cp_async_wait<P - 3>();
+                cta_barrier(blockDim.x);
+                issue();
+            }
         }
         cp_async_wait<0>();
         __syncthreads();
@@ -462,13 +456,13 @@ cudaError_t launch19_pass(const LaunchArgs& a, int grid, size_t smem, cudaStream
     void (*k)(const LaunchArgs);
     const bool w3 = PASS == 0 && !a.plain && a.wind3;
     if (a.use_one)
-        k = a.plain ? rd_step19_kernel<M, ST, true, true, PASS>
-            : w3    ? rd_step19_kernel<M, ST, true, false, PASS, PASS == 0>
-                    : rd_step19_kernel<M, ST, true, false, PASS>;
+        k = a.plain ? rd_march19_kernel<M, ST, true, true, PASS>
+            : w3    ? rd_march19_kernel<M, ST, true, false, PASS, PASS == 0>
+                    : rd_march19_kernel<M, ST, true, false, PASS>;
     else
-        k = a.plain ? rd_step19_kernel<M, ST, false, true, PASS>
-            : w3    ? rd_step19_kernel<M, ST, false, false, PASS, PASS == 0>
-                    : rd_step19_kernel<M, ST, false, false, PASS>;
+        k = a.plain ? rd_march19_kernel<M, ST, false, true, PASS>
+            : w3    ? rd_march19_kernel<M, ST, false, false, PASS, PASS == 0>
+                    : rd_march19_kernel<M, ST, false, false, PASS>;
     static size_t configured[6] = {0, 0, 0, 0, 0, 0};
     size_t& conf = configured[(a.plain ? 1 : w3 ? 2 : 0) + (a.use_one ? 3 : 0)];
     if (smem > conf) {

@@ -1,5 +1,5 @@
-"""The one- and two-step march kernel (rd_march_kernel) where it can go
-wrong: rows that end inside a vector or a tile, tiles and z-chunks that the
+"""The march kernels (rd_march_kernel: one or two steps per launch;
+rd_march19_kernel: the 19-point stencil) where they can go wrong: rows that end inside a vector or a tile, tiles and z-chunks that the
 grid does not fill, the smallest grids, wrapped and mirrored halos, held
 layers, wind and a source on the faces.  Every launch shape evaluates the
 same rounded operations, so results must equal the multi-level kernel's (an
@@ -57,3 +57,36 @@ def test_bits_equal_the_multi_level_kernel(kind, storage):
         for t in TUNINGS:
             got = run(t)
             assert np.array_equal(got.view(np.uint32), ref.view(np.uint32)), (shape, t)
+
+
+@pytest.mark.parametrize("kind", ["turing", "brusselator", "held", "air", "air_mixed",
+                                  "ch_table1", "plume"])
+def test_19_point_tilings_agree_and_match_the_oracle(kind):
+    import oracle
+    from paper_1004_0480_gb300.sim import Sim
+    oracle.build()
+    for shape in SHAPES:
+        if kind == "ch_table1":
+            cfg = W.with_(W.ch_table1(shape=shape), init="uniform_noise")
+        elif kind == "plume":
+            cfg = W.with_(W.plume(shape, src=(shape[0] - 1, 0, 0)), stencil=19,
+                          init="uniform_noise")
+        else:
+            # one diffusivity per species on this stencil
+            cfg = W.with_(problem(kind, shape), stencil=19)
+            cfg["D"] = [[d[0]] * 3 for d in cfg["D"]]
+        f = W.initial_fields(cfg)
+        ref = oracle.run(cfg, f, 5)
+        first = None
+        for t in (None, dict(tile_y=2, zchunk=1, graph=0), dict(tile_y=8, zchunk=3),
+                  dict(tile_y=14, zchunk=64)):
+            with Sim(cfg, tuning=t) as s:
+                s.set_fields(f)
+                s.step(5)
+                got = s.get_fields()
+            # FP32 rounding of 5 steps: some 20 roundings of 6e-8 a step,
+            # amplified at most a few times by the reactions
+            for a, b in zip(got, ref):
+                assert np.abs(a - b).max() <= 2e-5 * max(np.abs(b).max(), 1e-30), (shape, t)
+            first = got if first is None else first
+            assert np.array_equal(got.view(np.uint32), first.view(np.uint32)), (shape, t)
