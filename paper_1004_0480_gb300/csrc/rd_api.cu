@@ -948,6 +948,25 @@ bool is_device_ptr(const void* p) {
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// Whether the pack and unpack kernels may read or write the caller's ``n``
+// floats at p themselves: device memory of the current device, aligned, apart
+// from the context's own memory.  Anything else goes through the staging
+// field.
+bool kernel_may_touch(const rd_ctx* c, const void* p, size_t n) {
+    cudaPointerAttributes at{};
+    int dev = -1;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (at.type != cudaMemoryTypeDevice || at.device != dev) return false;
+    const char* lo = static_cast<const char*>(p);
+    const char* hi = lo + n * sizeof(float);
+    if (reinterpret_cast<uintptr_t>(p) % sizeof(float)) return false;
+    auto apart = [&](const char* m, size_t bytes) { return hi <= m || lo >= m + bytes; };
+    return apart(c->state, c->state_bytes) && apart(c->scratch, c->scratch_bytes);
+}
+
 std::mutex g_tune_mu;
 std::map<std::string, rd_tuning> g_tune_cache;
 bool g_tune_file_loaded = false;
@@ -1095,17 +1114,20 @@ rd_status rd_set_field(rd_ctx* c, int s, const float* src, size_t count) {
     const rd_config& g = c->cfg;
     const size_t n = (size_t)g.nx * g.ny * g.nz;
     if (count != n) return fail(c, RD_EINVAL, "count %zu != nx*ny*nz = %zu", count, n);
-    const bool dev = is_device_ptr(src);
-    RD_CUDA(c, cudaMemcpyAsync(c->staging, src, n * sizeof(float),
-                               dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->stream));
+    const bool direct = kernel_may_touch(c, src, n);
+    if (!direct)
+        RD_CUDA(c, cudaMemcpyAsync(c->staging, src, n * sizeof(float),
+                                   is_device_ptr(src) ? cudaMemcpyDeviceToDevice
+                                                      : cudaMemcpyHostToDevice,
+                                   c->stream));
     float hv[6];
     unsigned m = 0;
     for (int f = 0; f < 6; ++f) {
         hv[f] = (float)g.bc_value[s][f];
         if (g.bc[s][f] == RD_BC_DIRICHLET) m |= 1u << f;
     }
-    cudaError_t e = launch_pack(c->staging, field_ptr(c, c->cur, s), g.storage, g.nx, g.ny, g.nz,
-                                c->pitch, m, hv, c->stream);
+    cudaError_t e = launch_pack(direct ? src : c->staging, field_ptr(c, c->cur, s), g.storage, g.nx,
+                                g.ny, g.nz, c->pitch, m, hv, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "pack kernel");
     c->launches++;
     RD_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -1120,13 +1142,16 @@ rd_status rd_get_field(rd_ctx* c, int s, float* dst, size_t count) {
     const rd_config& g = c->cfg;
     const size_t n = (size_t)g.nx * g.ny * g.nz;
     if (count != n) return fail(c, RD_EINVAL, "count %zu != nx*ny*nz = %zu", count, n);
-    cudaError_t e = launch_unpack(field_ptr(c, c->cur, s), c->staging, g.storage, g.nx, g.ny,
-                                  g.nz, c->pitch, c->stream);
+    const bool direct = kernel_may_touch(c, dst, n);
+    cudaError_t e = launch_unpack(field_ptr(c, c->cur, s), direct ? dst : c->staging, g.storage,
+                                  g.nx, g.ny, g.nz, c->pitch, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "unpack kernel");
     c->launches++;
-    const bool dev = is_device_ptr(dst);
-    RD_CUDA(c, cudaMemcpyAsync(dst, c->staging, n * sizeof(float),
-                               dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
+    if (!direct)
+        RD_CUDA(c, cudaMemcpyAsync(dst, c->staging, n * sizeof(float),
+                                   is_device_ptr(dst) ? cudaMemcpyDeviceToDevice
+                                                      : cudaMemcpyDeviceToHost,
+                                   c->stream));
     RD_CUDA(c, cudaStreamSynchronize(c->stream));
     return RD_OK;
 }
