@@ -579,6 +579,7 @@ PlaneCost plane_cost(const rd_config& g, int T) {
                : g.nspecies == 2 ? PlaneCost{0.0, 0.6, 0.0146}
                                  : PlaneCost{0.0, 0.9, 0.0300};
     }
+    if (is_ch(g.model)) return {0.21, 0.0, 0.0290};
     switch (g.nspecies) {
     case 1: return T == 2 ? PlaneCost{0.20, 0.0, 0.0135} : PlaneCost{0.17, 0.0, 0.0085};
     case 2:
@@ -601,10 +602,8 @@ constexpr double kLaunchUs = 2.4;
 rd_tuning default_plan(const rd_config& g, const rd_tuning& t1, int maxT) {
     rd_tuning best = t1;
     const int sten = stencil_of(g);
-    if (is_ch(g.model) && sten == 7) {   // no plan: the tuning as it is
-        best.tsteps = 0;
-        return best;
-    }
+    // the march kernel's T = 2 has no Cahn-Hilliard form
+    if (is_ch(g.model)) maxT = 1;
     const int sms = num_sms();
     double best_cost = -1.0;
     for (int T = 1; T <= std::min(maxT, max_tsteps(g)); ++T)
@@ -630,7 +629,7 @@ rd_tuning default_plan(const rd_config& g, const rd_tuning& t1, int maxT) {
                 last = zc;
                 const long long items = cols * tiles(g.nz, zc);
                 const long long full = items / slots, rest = items % slots;
-                const double planes = zc + 2 * (T - 1) + 1;
+                const double planes = zc + 2 * (T - 1) + 1 + (is_ch(g.model) && sten == 7 ? 2 : 0);
                 const double us =
                     planes * (full * plane_us(occ) + plane_us(tiles((int)rest, sms)));
                 const double cost = (kLaunchUs * kernels_per_step(g) + us) / T;

@@ -127,8 +127,15 @@ template <class M, class ST, int T> struct LayoutM {
     }
 };
 
-// How one vector of a two-step launch is fetched: as make_fetch, but rows
-// beyond a zero-flux y face are mirror images, vectors beyond a zero-flux x
+// Mirror extension: -1-i for i < 0, 2n-1-i for i >= n; clamped so that
+// positions outside the grid by more than n (never stored) stay in bounds.
+__device__ __forceinline__ int mirror_index(int i, int n) {
+    const int m = i < 0 ? -1 - i : (i >= n ? 2 * n - 1 - i : i);
+    return min(max(m, 0), n - 1);
+}
+
+// How one vector of a march is fetched: rows beyond a zero-flux y face are
+// mirror images, vectors beyond a zero-flux x
 // face are not fetched, and the last vector of a row that ends inside it is
 // copied whole (its tail is the row's padding, never read).
 template <class ST>

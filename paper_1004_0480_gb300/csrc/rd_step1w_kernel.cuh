@@ -86,7 +86,8 @@ template <> struct Vec8<__nv_bfloat16> {
     }
 };
 
-// How one 8-cell vector is fetched (see make_fetch; the same rules).
+// How one 8-cell vector is fetched: rows beyond a zero-flux face are the face
+// row, cells beyond one in x clamped.
 template <class ST>
 __device__ __forceinline__ Fetch make_fetch8(int yrow, int xs, int nx, int ny, int pitch, bool px,
                                              bool py, int soff_elems) {

@@ -4,7 +4,7 @@
 // shape gives the same bits: rd_step_kernel (T steps per launch, any tile
 // height, described here), rd_march_kernel (one or two steps per launch, even
 // heights, models without Cahn-Hilliard), rd_step1w_kernel (one step, 8 cells
-// per thread) and rd_stepch_kernel (one step, the Cahn-Hilliard models); the
+// per thread) and rd_marchch_kernel (one step, the Cahn-Hilliard models); the
 // others are described where they are defined.
 //
 // rd_step_kernel: one launch advances T steps of eq. (5) for every species
@@ -540,7 +540,10 @@ __device__ __forceinline__ unsigned z_faces(int q, int nz) {
 // per-cell tests run only where a held face is touched
 __device__ __forceinline__ void held_layers_at(const InstDesc& sd, int s, unsigned faces, int xs,
                                                int y, int q, float (&o)[kVEC]) {
-    if (sd.held_mask[s] & faces) held_layers(sd, s, xs, y, q, o);
+    if (sd.held_mask[s] & faces) {
+        asm volatile("");   // keep the branch: few vectors touch a held face
+        held_layers(sd, s, xs, y, q, o);
+    }
 }
 
 // First-order upwind along one axis with Courant number cu = u dt / h:
@@ -828,93 +831,15 @@ __global__ void __launch_bounds__(kMaxThreads, 2) rd_step_kernel(const __grid_co
     }
 }
 
-// How one vector is fetched: 1 = one async copy, 2 = element by element
-// (wrapped x, or clamped x for a vector straddling a zero-flux face), 0 =
-// nothing (a vector wholly outside a zero-flux x face, or a row outside a
-// face that is never read: the kernels take the face cell from the
-// thread's own vector instead, see xface_offsets).
+// How one vector is fetched: 1 = one async copy, 2 = element by element (a
+// vector that wraps round a periodic x axis; in the 8-cell kernel also one
+// straddling a zero-flux face), 0 = nothing.
 struct Fetch {
     int mode;
     int goff;    // element offset of row + x within a plane
     int soff;    // byte offset of the position within a plane buffer
     int xs;      // global x of the vector's first element (unwrapped)
 };
-
-template <class ST>
-__device__ __forceinline__ Fetch make_fetch(int yrow, int xs, int nx, int ny, int pitch, bool px,
-                                            bool py, int soff_elems, bool clamp) {
-    Fetch f{0, 0, soff_elems * (int)sizeof(ST), xs};
-    int yw = yrow;
-    if (py) {
-        yw = wrapi(yrow, ny);
-    } else if (yrow < 0 || yrow >= ny) {
-        if (!clamp) return f;                     // never read
-        yw = yrow < 0 ? 0 : ny - 1;               // ghost row = face row
-    }
-    const int row = yw * pitch;
-    if (xs >= 0 && xs + kVEC <= nx) {
-        f.mode = 1;
-        f.goff = row + xs;
-    } else if (px) {
-        const int xw = wrapi(xs, nx);
-        if (xw % kVEC == 0 && xw + kVEC <= nx) { f.mode = 1; f.goff = row + xw; }
-        else { f.mode = 2; f.goff = row; }
-    } else if (clamp) {
-        if (xs < nx && xs + kVEC > 0) {           // straddles the face: ghost
-            f.mode = 2;                           // cells = face cell
-            f.goff = row;
-        }
-    } else if (xs >= 0 && xs < nx) {
-        f.mode = 1;                               // last vector: tail in the row padding
-        f.goff = row + xs;
-    }
-    return f;
-}
-
-// one fetch of every species of a plane; ``elems`` is true where mode 2 can
-// occur (zero-flux x faces, periodic x with nx not a multiple of 4); its
-// element copies are 4-byte async copies for FP32, plain loads for BF16
-template <class ST, int S>
-__device__ __forceinline__ void fetch_all(const Fetch& f, unsigned char* plane_buf, int pe_bytes,
-                                          const ST* gplane, long long fstride, int nx,
-                                          bool elems, bool px, const InstDesc& sd) {
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-        const ST* src = gplane + s * fstride + f.goff;
-        const int ok =
-            f.mode == 1 && RD_DBG_GLOBAL(sd, src, 4 * (int)sizeof(ST), kSiteCopySrc);
-        Store<ST>::cp_async_if(reinterpret_cast<ST*>(plane_buf + s * pe_bytes + f.soff), src, ok);
-    }
-    if (elems && f.mode == 2) {
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-            ST* d = reinterpret_cast<ST*>(plane_buf + s * pe_bytes + f.soff);
-#pragma unroll
-            for (int e = 0; e < kVEC; ++e) {
-                const int x = f.xs + e;
-                const int xi = px ? wrapi(x, nx) : (x < 0 ? 0 : (x >= nx ? nx - 1 : x));
-                const ST* src = gplane + s * fstride + f.goff + xi;
-                if (RD_DBG_GLOBAL(sd, src, (int)sizeof(ST), kSiteCopySrc))
-                    Store<ST>::cp_async_elem(d + e, src);
-            }
-        }
-    }
-}
-
-// Byte offsets, from a thread's own vector in a plane buffer, of the x
-// neighbours beside it: the element left of element 0 and right of element
-// 3.  At a zero-flux x face the ghost there equals the face cell, which is
-// the thread's own element 0 (left face) or 3 (a vector ending at the right
-// face), so those offsets point into the own vector and the vectors outside
-// the face are never copied (element-by-element copies of them had cost a
-// quarter of the step).  A vector straddling the right face (nx not a
-// multiple of 4) holds its clamped ghosts itself.
-template <class ST>
-__device__ __forceinline__ void xface_offsets(int xs, int nx, bool px, int& loff, int& roff) {
-    constexpr int EB = (int)sizeof(ST);
-    loff = (!px && xs == 0) ? 0 : -EB;
-    roff = (!px && xs + kVEC == nx) ? (kVEC - 1) * EB : kVEC * EB;
-}
 
 template <class ST>
 __device__ __forceinline__ void lds_vec(const unsigned char* p, float (&v)[kVEC]) {
@@ -928,8 +853,8 @@ __device__ __forceinline__ float lds_one(const unsigned char* p) {
 }  // namespace rdk
 
 #include "rd_step1w_kernel.cuh"
-#include "rd_stepch_kernel.cuh"
 #include "rd_march_kernel.cuh"
+#include "rd_stepch_kernel.cuh"
 
 namespace rdk {
 
@@ -947,7 +872,7 @@ cudaError_t launch_one(const LaunchArgs& a, int grid, size_t smem, cudaStream_t 
     // which kernel, and its slot in ``configured`` below
     int variant = 0;
     if constexpr (T == 1 && M::CH) {
-        k = a.plain ? rd_stepch_kernel<M, ST, ONE, true> : rd_stepch_kernel<M, ST, ONE, false>;
+        k = a.plain ? rd_marchch_kernel<M, ST, ONE, true> : rd_marchch_kernel<M, ST, ONE, false>;
         threads = LayoutCH<ST>::threads(a.ty);
         variant = a.plain ? 1 : 0;
     } else if constexpr (T == 1) {

@@ -1,5 +1,5 @@
 """The march kernels (rd_march_kernel: one or two steps per launch;
-rd_march19_kernel: the 19-point stencil) where they can go wrong: rows that end inside a vector or a tile, tiles and z-chunks that the
+rd_march19_kernel: the 19-point stencil; rd_marchch_kernel: Cahn-Hilliard) where they can go wrong: rows that end inside a vector or a tile, tiles and z-chunks that the
 grid does not fill, the smallest grids, wrapped and mirrored halos, held
 layers, wind and a source on the faces.  Every launch shape evaluates the
 same rounded operations, so results must equal the multi-level kernel's (an
@@ -90,3 +90,32 @@ def test_19_point_tilings_agree_and_match_the_oracle(kind):
                 assert np.abs(a - b).max() <= 2e-5 * max(np.abs(b).max(), 1e-30), (shape, t)
             first = got if first is None else first
             assert np.array_equal(got.view(np.uint32), first.view(np.uint32)), (shape, t)
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+@pytest.mark.parametrize("kind", ["front", "periodic_front", "source_front", "table1"])
+def test_cahn_hilliard_bits_equal_the_multi_level_kernel(kind, storage):
+    from paper_1004_0480_gb300.sim import Sim
+    for shape in SHAPES:
+        if kind == "table1":
+            cfg = W.with_(W.ch_table1(shape=shape, dt=0.001, stencil=7), init="uniform_noise")
+        else:
+            cfg = W.with_(W.ch_front(shape=shape), init="uniform_noise")
+        if kind == "periodic_front":
+            cfg = W.with_(cfg, bc=[[P] * 6] * 3)
+        if kind == "source_front":          # the general variant
+            nx, ny, nz = shape
+            cfg = W.with_(cfg, source=dict(x=nx - 1, y=ny - 1, z=0, species=1, rate=2.0),
+                          D=[[1.0, 0.5, 0.25], [0.1] * 3, [0.0] * 3])
+        f = W.initial_fields(cfg)
+
+        def run(tuning):
+            with Sim(cfg, storage, tuning=tuning) as s:
+                s.set_fields(f)
+                s.step(4)
+                return s.get_fields()
+        ref = run(dict(tsteps=2, tile_y=5, zchunk=3))
+        for t in (None, dict(tsteps=1, tile_y=12, zchunk=4), dict(tsteps=1, tile_y=5, zchunk=1),
+                  dict(tsteps=1, tile_y=26, zchunk=2, graph=0)):
+            got = run(t)
+            assert np.array_equal(got.view(np.uint32), ref.view(np.uint32)), (shape, t)
