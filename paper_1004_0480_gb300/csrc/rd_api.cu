@@ -588,8 +588,10 @@ PlaneCost plane_cost(const rd_config& g, int T) {
     default: return T == 2 ? PlaneCost{0.40, 0.0, 0.0770} : PlaneCost{0.30, 0.0, 0.0340};
     }
 }
-// launch gap and pipeline fill of a launch (replayed from a graph)
-constexpr double kLaunchUs = 2.4;
+// launch gap and pipeline fill of a launch (replayed from a graph), and the
+// least a plane takes however few rows an SM holds (copies, barrier, the
+// chain of one update)
+constexpr double kLaunchUs = 1.9, kPlaneUs = 0.45;
 
 // What a context steps with while its tuning is the default one: the tile
 // height, z-chunk and steps per launch (at most ``maxT``) of the least
@@ -618,7 +620,7 @@ rd_tuning default_plan(const rd_config& g, const rd_tuning& t1, int maxT) {
             const PlaneCost pc = plane_cost(g, T);
             // an SM's time per plane with ``ctas`` work items on it
             auto plane_us = [&](int ctas) {
-                return ctas ? pc.a + pc.a1 / ctas + pc.b * ctas * ty : 0.0;
+                return ctas ? std::max(kPlaneUs, pc.a + pc.a1 / ctas + pc.b * ctas * ty) : 0.0;
             };
             const long long cols = (long long)tiles(g.nx, kTileW) * tiles(g.ny, ty);
             const long long slots = (long long)occ * sms;

@@ -338,6 +338,7 @@ rd_march_kernel(const __grid_constant__ LaunchArgs a) {
     const int own0 = kVEC * EB + (t.r + T - 1) * RM::ROWB + t.v * kVEC * EB;
     const int own1 = (int)LY::ring_bytes(TY) + kVEC * EB + t.r * RM::ROWB + t.v * kVEC * EB;
 
+    if constexpr (!ONE) chain_wait();   // the batch's counters are read first
     int cur_inst = -1;
     if (tid == 0) s_inst = 0;
     for (long long item = first_item<ONE>(a, s_item); item < a.nitems;
@@ -369,6 +370,7 @@ rd_march_kernel(const __grid_constant__ LaunchArgs a) {
         const unsigned xyf = xy_faces(xs, y, nx, ny);
         const bool src_col = sd.src_s >= 0 && yw == sd.src_y;
         const bool elems = sd.wrap_elems;
+        if constexpr (ONE) chain_wait();   // nothing above reads what a launch writes
         float cy = 0.0f, cz = 0.0f;                   // 3-D wind
         if constexpr (W3) wind3d(sd, lin, local, cy, cz);
         // what the thread copies of every plane, offsets from its own vector:
@@ -534,6 +536,7 @@ rd_march_kernel(const __grid_constant__ LaunchArgs a) {
             body(e, C0, A0, B0, C1, A1, B1);
             if (++e == z1 + T - 1) break;
         }
+        if (ONE && item + gridDim.x >= a.nitems) chain_release();   // the last item
         cp_async_wait<0>();
         __syncthreads();
     }

@@ -182,6 +182,7 @@ rd_march19_kernel(const __grid_constant__ LaunchArgs a) {
     int4* const hfetch = reinterpret_cast<int4*>(smem + RING * SLOTB);
     const int mu_own = NS * SPB + t.v * kVEC * (4 - EB);     // from the own vector
 
+    if constexpr (!ONE) chain_wait();   // the batch's counters are read first
     int cur_inst = -1;
     if (tid == 0) s_inst = 0;
     for (long long item = first_item<ONE>(a, s_item); item < a.nitems;
@@ -222,6 +223,7 @@ rd_march19_kernel(const __grid_constant__ LaunchArgs a) {
         for (int s = 0; s < S; ++s) k6[s] = __fdiv_rn(sd.kx[s], 6.0f);
         if constexpr (PASS == 1) k6[0] = __fdiv_rn(sd.p[2], 6.0f);
         if constexpr (PASS == 2) k6[2] = __fdiv_rn(sd.p[1], 6.0f);
+        if constexpr (ONE) chain_wait();   // nothing above reads what a launch writes
         float cy = 0.0f, cz = 0.0f;                   // 3-D wind
         if constexpr (W3 && PASS == 0) wind3d(sd, lin, local, cy, cz);
         // what the thread copies of every plane: its own vector, element
@@ -441,6 +443,7 @@ rd_march19_kernel(const __grid_constant__ LaunchArgs a) {
                 issue();
             }
         }
+        if (ONE && item + gridDim.x >= a.nitems) chain_release();   // the last item
         cp_async_wait<0>();
         __syncthreads();
     }
@@ -474,8 +477,7 @@ cudaError_t launch19_pass(const LaunchArgs& a, int grid, size_t smem, cudaStream
     const int threads = Layout19<M, ST, PASS>::threads(a.ty);
     if (threads > kMaxThreads) return cudaErrorInvalidConfiguration;
     if (occ) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, threads, smem);
-    k<<<grid, threads, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k, a, grid, threads, smem, st);
 }
 
 template <class M>

@@ -871,6 +871,7 @@ cudaError_t launch_one(const LaunchArgs& a, int grid, size_t smem, cudaStream_t 
     int threads = 0;
     // which kernel, and its slot in ``configured`` below
     int variant = 0;
+    bool chained = true;       // march kernels wait for the launch before them
     if constexpr (T == 1 && M::CH) {
         k = a.plain ? rd_marchch_kernel<M, ST, ONE, true> : rd_marchch_kernel<M, ST, ONE, false>;
         threads = LayoutCH<ST>::threads(a.ty);
@@ -887,6 +888,7 @@ cudaError_t launch_one(const LaunchArgs& a, int grid, size_t smem, cudaStream_t 
                           : rd_step1w_kernel<M, ST, ONE, false, false>;
             threads = Layout1w<M, ST>::threads(a.ty);
             variant = a.plain ? 1 : a.wind3 ? 2 : 3;
+            chained = false;
         } else if (lean) {
             k = a.plain   ? rd_march_kernel<M, ST, 1, ONE, true, false>
                 : a.wind3 ? rd_march_kernel<M, ST, 1, ONE, false, true>
@@ -896,12 +898,15 @@ cudaError_t launch_one(const LaunchArgs& a, int grid, size_t smem, cudaStream_t 
         } else {
             k = rd_step_kernel<M, ST, T, ONE>;
             threads = Layout<M, ST, T>::threads(a.ty);
+            chained = false;
         }
     } else {
         k = rd_step_kernel<M, ST, T, ONE>;
         threads = Layout<M, ST, T>::threads(a.ty);
+        chained = false;
         if constexpr (T == 2 && !M::CH)
             if (two_step<M, ST>(T, a.ty)) {
+                chained = true;
                 k = a.plain ? rd_march_kernel<M, ST, 2, ONE, true, false>
                             : rd_march_kernel<M, ST, 2, ONE, false, false>;
                 threads = LayoutM<M, ST, 2>::threads(a.ty);
@@ -919,6 +924,7 @@ cudaError_t launch_one(const LaunchArgs& a, int grid, size_t smem, cudaStream_t 
     }
     if (threads > kMaxThreads) return cudaErrorInvalidConfiguration;
     if (occ) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, threads, smem);
+    if (chained) return launch_chained(k, a, grid, threads, smem, st);
     k<<<grid, threads, smem, st>>>(a);
     return cudaGetLastError();
 }

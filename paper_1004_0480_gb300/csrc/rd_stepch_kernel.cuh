@@ -78,6 +78,7 @@ rd_marchch_kernel(const __grid_constant__ LaunchArgs a) {
     const int own0 = kVEC * EB + (t.r + 1) * RM::ROWB + t.v * kVEC * EB;
     const int ownm = (int)LY::state_bytes(TY) + (kVEC + t.v * kVEC) * 4 + t.r * RMU::ROWB;
 
+    if constexpr (!ONE) chain_wait();   // the batch's counters are read first
     int cur_inst = -1;
     if (tid == 0) s_inst = 0;
     for (long long item = first_item<ONE>(a, s_item); item < a.nitems;
@@ -115,6 +116,7 @@ rd_marchch_kernel(const __grid_constant__ LaunchArgs a) {
             fx = make_fetch_h<ST>(t.r ? y + 1 : y - 1, xs, nx, ny, pitch, px, py,
                                   (t.r ? RM::ROWB : -RM::ROWB) + 2 * RM::SPB);
 
+        if constexpr (ONE) chain_wait();   // nothing above reads what a launch writes
         // planes z0-2 .. z1+1 are copied; the next one to slot_ld
         PlaneFeed feed(z0 - 2, nz, pz);
         const int slot_end = own0 + RING * SLOTB;
@@ -252,6 +254,7 @@ rd_marchch_kernel(const __grid_constant__ LaunchArgs a) {
             body(e, AC, AA, AB, CC, CA, CB, MX, MA, MB);
             if (++e == z1 + 1) break;
         }
+        if (ONE && item + gridDim.x >= a.nitems) chain_release();   // the last item
         cp_async_wait<0>();
         __syncthreads();
     }
