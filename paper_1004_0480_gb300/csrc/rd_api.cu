@@ -191,9 +191,11 @@ int max_tsteps(const rd_config& g) {
 
 // CTAs per SM for a variant (cached).
 bool plain_problem(const rd_config& g);
-// kernel variant of a problem: 1 branch-free, 2 with the 3-D wind, else 0
+bool windx_problem(const rd_config& g);
+// kernel variant of a problem: 1 branch-free, 2 with the 3-D wind, 3 with wind
+// along +x (or none) and anisotropic species, else 0
 int variant_code(const rd_config& g) {
-    return plain_problem(g) ? 1 : g.wind_kind == RD_WIND_3D ? 2 : 0;
+    return plain_problem(g) ? 1 : g.wind_kind == RD_WIND_3D ? 2 : windx_problem(g) ? 3 : 0;
 }
 
 int occupancy(int model, int storage, int T, int ty, int regcap = 0, int plain = 0,
@@ -208,9 +210,10 @@ int occupancy(int model, int storage, int T, int ty, int regcap = 0, int plain =
     LaunchArgs dummy{};
     dummy.use_one = 1;
     dummy.regcap = regcap;
-    // plain: 0 the general variant, 1 the branch-free one, 2 the 3-D wind one
+    // plain: a variant_code
     dummy.plain = plain == 1;
     dummy.wind3 = plain == 2;
+    dummy.windx = plain == 3;
     dummy.ty = ty;
     dummy.vw = vw_of(tq);
     const size_t smem = smem_of(model, storage, T, ty, stencil, tq);
@@ -742,6 +745,24 @@ bool plain_problem(const rd_config& g) {
     return true;
 }
 
+// No held layer, wind along +x (or none) and every species anisotropic: the
+// one-step march kernel's kWindX variant applies.
+bool windx_problem(const rd_config& g) {
+    if (is_ch(g.model) || stencil_of(g) == 19 || g.wind_kind == RD_WIND_3D) return false;
+    if (g.wind_kind != RD_WIND_NONE && !(g.wind_u0 >= 0.0)) return false;
+    for (int s = 0; s < g.nspecies; ++s) {
+        for (int f = 0; f < 6; ++f)
+            if (g.bc[s][f] == RD_BC_DIRICHLET) return false;
+        // as the kernels see them (fill_desc)
+        const double ih2 = 1.0 / (g.h * g.h);
+        const float kx = (float)(g.D[s][0] * g.dt * ih2);
+        const float ky = (float)(g.D[s][1] * g.dt * ih2);
+        const float kz = (float)(g.D[s][2] * g.dt * ih2);
+        if (kx == ky && kx == kz) return false;
+    }
+    return true;
+}
+
 rd_status upload_desc(rd_ctx* c) {
     if (!c->desc_dirty) return RD_OK;
     fill_desc(c, c->desc, c->tun);
@@ -802,6 +823,7 @@ rd_status launch_ctx(rd_ctx* c, int T, int parity, cudaStream_t st, Use use = Us
     a.regcap = t.regcap;
     a.plain = plain_problem(c->cfg);
     a.wind3 = c->cfg.wind_kind == RD_WIND_3D;
+    a.windx = windx_problem(c->cfg);
     a.vw = vw_of(t.tile_q);
     a.ty = t.tile_y;
     if (c->kernel == RD_KERNEL_RESIDENT) {
@@ -827,7 +849,7 @@ rd_status launch_ctx(rd_ctx* c, int T, int parity, cudaStream_t st, Use use = Us
     const size_t sm = smem_of(c->cfg.model, c->cfg.storage, T, a.ty, sten, t.tile_q);
     const int occ = std::max(
         1, occupancy(c->cfg.model, c->cfg.storage, T, a.ty, a.regcap,
-                     a.plain ? 1 : a.wind3 ? 2 : 0, sten, t.tile_q));
+                     variant_code(c->cfg), sten, t.tile_q));
     const long long grid = std::min<long long>(a.nitems, (long long)occ * num_sms());
     cudaError_t e =
         launch_model(c->cfg.model, c->cfg.storage, T, a, (int)grid, sm, st, nullptr, sten);

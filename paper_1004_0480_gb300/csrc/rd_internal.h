@@ -65,6 +65,8 @@ struct LaunchArgs {
                                // wind, and isotropic diffusivities
     int wind3;                 // some instance has the 3-D wind (kernels take
                                // the variant with upwind along y and z)
+    int windx;                 // the instance has no held layer, wind along +x
+                               // or none, and every species anisotropic
     int vw;                    // cells per thread of the one-step 7-point
                                // kernel: 4 (16 threads per tile row) or 8
     unsigned long long* work;  // batches that pull items: work[0] the

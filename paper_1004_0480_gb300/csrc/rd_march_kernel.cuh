@@ -107,7 +107,7 @@ template <class M, class ST, int T> struct LayoutM {
     //                           T = 1: 366 (128) 371 (96) 387 (80) 291 (64)
     //   the same in BF16, T = 2: 441 (128) 362 (112) 312 (96)
     //                     T = 1: 457 (128) 451 (96) 401 (80) 296 (64)
-    //   air 512 x 512 x 64 FP32, T = 1: 198 (128) 160 (96) 133 (80)
+    //   air 512 x 512 x 64 FP32, T = 1: 253 (128) 249 (112) 215 (96)
     // The general and batch variants take 16 more.
     static constexpr int regs(bool lean) {
         if (S == 3 || (S == 2 && sizeof(ST) == 2)) return 128;
@@ -295,18 +295,27 @@ struct PlaneFeed {
     }
 };
 
-// PLAIN: no held layer, point source or wind, every species isotropic.  W3:
-// the 3-D wind (upwind along y and z too; T = 1, never with PLAIN).
-template <class M, class ST, int T, bool ONE, bool PLAIN, bool W3>
+// What a problem may have beside reactions and diffusion, so that the kernel
+// tests for nothing else: kPlain: no held layer, point source or wind, every
+// species isotropic; kWindX: no held layer, wind along +x or none, every
+// species anisotropic (the air problem, 512 x 512 x 64: 253 GLUPS, 0.90 of
+// the HBM copy rate, against 197 in the general variant); kWind3: the 3-D wind (upwind along y
+// and z too; T = 1); kGeneral: anything else.
+enum MarchVar { kGeneral, kPlain, kWind3, kWindX };
+
+template <class M, class ST, int T, bool ONE, int VAR>
 __global__ void
 #ifdef RDM_ATTR
 RDM_ATTR
 #else
-__maxnreg__((LayoutM<M, ST, T>::regs(ONE && PLAIN)))
+__maxnreg__((LayoutM<M, ST, T>::regs(ONE && VAR == kPlain)))
 #endif
 rd_march_kernel(const __grid_constant__ LaunchArgs a) {
     static_assert(T == 1 || T == 2, "one or two steps per launch");
-    static_assert(!W3 || (T == 1 && !PLAIN), "the 3-D wind steps once per launch");
+    static_assert(VAR != kWindX || T == 1, "the Courant number is read one plane ahead");
+    constexpr bool PLAIN = VAR == kPlain;
+    constexpr bool W3 = VAR == kWind3;
+    static_assert(!W3 || T == 1, "the 3-D wind steps once per launch");
     using LY = LayoutM<M, ST, T>;
     using RM = typename LY::RM;
     constexpr int S = M::S;
@@ -407,7 +416,7 @@ rd_march_kernel(const __grid_constant__ LaunchArgs a) {
                 unsigned char* const d = smem + slot_ld;
 #pragma unroll
                 for (int k = 0; k < NF; ++k) {
-                    if (k > 0 && inner_warp) break;
+                    if (k == 0 || !inner_warp)   // (no break: f stays in registers)
 #pragma unroll
                     for (int s = 0; s < S; ++s) {
                         const ST* gs = g + f[k].goff + s * fstride;
@@ -430,6 +439,10 @@ rd_march_kernel(const __grid_constant__ LaunchArgs a) {
 #pragma unroll 1
         for (int j = 0; j < P; ++j) issue();
 
+        // kWindX: the Courant number of the plane being advanced and of the
+        // next, loaded a plane ahead
+        float cxq = 0.0f, cxn = 0.0f;
+        if constexpr (VAR == kWindX) cxn = courant_at(sd, sd.courant, z0);
         // one step of the position's cells in plane q (mapped index zw):
         // centres cen, z neighbours zm / zp, x and y neighbours around ``p``
         auto advance = [&](const float(&zm)[S][kVEC], const float(&cen)[S][kVEC],
@@ -437,7 +450,7 @@ rd_march_kernel(const __grid_constant__ LaunchArgs a) {
                            float(&o)[S][kVEC]) {
             float inc[S][kVEC];
             react4<M>(sd, cen, inc);
-            const float cx = PLAIN ? 0.0f : courant_at(sd, sd.courant, zw);
+            const float cx = PLAIN || VAR == kWindX ? 0.0f : courant_at(sd, sd.courant, zw);
             const bool src_here = src_col && zw == sd.src_z;
             const unsigned faces = xyf | z_faces(q, nz);
 #pragma unroll
@@ -449,6 +462,26 @@ rd_march_kernel(const __grid_constant__ LaunchArgs a) {
                 sides.get<ST>(cen[s], ps, xm, xp);
                 if constexpr (PLAIN) {
                     euler4_iso(cen[s], xm, xp, ym, yp, zm[s], zp[s], sd.kx[s], inc[s], o[s]);
+                } else if constexpr (VAR == kWindX) {
+                    // behind the loads, on a copy of its own: a branch ahead of
+                    // them holds them up, and the species' writes merged into
+                    // one would be indexed in local memory
+                    float in[kVEC];
+#pragma unroll
+                    for (int i = 0; i < kVEC; ++i) in[i] = inc[s][i];
+                    if (src_here && s == sd.src_s) {
+#pragma unroll
+                        for (int i = 0; i < kVEC; ++i)
+                            if ((px ? wrapi(xs + i, nx) : xs + i) == sd.src_x)
+                                in[i] = __fadd_rn(in[i], sd.src_amt);
+                    }
+                    if (cxq != 0.0f) {
+#pragma unroll
+                        for (int i = 0; i < kVEC; ++i)
+                            in[i] = __fmaf_rn(-cxq, __fsub_rn(cen[s][i], xm[i]), in[i]);
+                    }
+                    euler4_aniso(cen[s], xm, xp, ym, yp, zm[s], zp[s], sd.kx[s], sd.ky[s],
+                                 sd.kz[s], in, o[s]);
                 } else {
                     species_core(sd, s, cen[s], xm, xp, ym, yp, zm[s], zp[s], inc[s], cx, src_here,
                                  px, xs, o[s], cy, cz);
@@ -503,6 +536,10 @@ rd_march_kernel(const __grid_constant__ LaunchArgs a) {
             }
             issue();   // after the reads of plane e - 1, whose slot it refills
             if constexpr (T == 1) {
+                if constexpr (VAR == kWindX) {
+                    cxq = cxn;
+                    cxn = courant_at(sd, sd.courant, min(e + 1, nz - 1));
+                }
                 if (inner_warp) {
                     float o[S][kVEC];
                     advance(m0, c0, p0, smem + s1, e, e, o);

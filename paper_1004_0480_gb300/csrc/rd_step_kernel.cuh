@@ -310,6 +310,20 @@ __device__ __forceinline__ void euler4_iso(const float (&c)[kVEC], const float (
                                       vadd(pair_of(zm, h), pair_of(zp, h)), k, pair_of(inc, h)));
 }
 
+// 4 cells of euler_cell
+__device__ __forceinline__ void euler4_aniso(const float (&c)[kVEC], const float (&xm)[kVEC],
+                                             const float (&xp)[kVEC], const float (&ym)[kVEC],
+                                             const float (&yp)[kVEC], const float (&zm)[kVEC],
+                                             const float (&zp)[kVEC], float kx, float ky, float kz,
+                                             const float (&inc)[kVEC], float (&o)[kVEC]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        set_pair(o, h, euler_cell(pair_of(c, h), xsum_of(xm, xp, h),
+                                  vadd(pair_of(ym, h), pair_of(yp, h)),
+                                  vadd(pair_of(zm, h), pair_of(zp, h)), kx, ky, kz,
+                                  pair_of(inc, h)));
+}
+
 // 4 cells of a species with any diffusivities: euler_cell_iso where they are
 // equal, else euler_cell
 __device__ __forceinline__ void euler4(const float (&c)[kVEC], const float (&xm)[kVEC],
@@ -317,16 +331,8 @@ __device__ __forceinline__ void euler4(const float (&c)[kVEC], const float (&xm)
                                        const float (&yp)[kVEC], const float (&zm)[kVEC],
                                        const float (&zp)[kVEC], float kx, float ky, float kz,
                                        const float (&inc)[kVEC], float (&o)[kVEC]) {
-    if (kx == ky && kx == kz) {
-        euler4_iso(c, xm, xp, ym, yp, zm, zp, kx, inc, o);
-        return;
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-        set_pair(o, h, euler_cell(pair_of(c, h), xsum_of(xm, xp, h),
-                                  vadd(pair_of(ym, h), pair_of(yp, h)),
-                                  vadd(pair_of(zm, h), pair_of(zp, h)), kx, ky, kz,
-                                  pair_of(inc, h)));
+    if (kx == ky && kx == kz) euler4_iso(c, xm, xp, ym, yp, zm, zp, kx, inc, o);
+    else euler4_aniso(c, xm, xp, ym, yp, zm, zp, kx, ky, kz, inc, o);
 }
 
 // mu = g(c) - p[2] (sum of 6 neighbours - 6 c) of the thread's 4 cells
@@ -890,11 +896,15 @@ cudaError_t launch_one(const LaunchArgs& a, int grid, size_t smem, cudaStream_t 
             variant = a.plain ? 1 : a.wind3 ? 2 : 3;
             chained = false;
         } else if (lean) {
-            k = a.plain   ? rd_march_kernel<M, ST, 1, ONE, true, false>
-                : a.wind3 ? rd_march_kernel<M, ST, 1, ONE, false, true>
-                          : rd_march_kernel<M, ST, 1, ONE, false, false>;
+            k = a.plain   ? rd_march_kernel<M, ST, 1, ONE, kPlain>
+                : a.wind3 ? rd_march_kernel<M, ST, 1, ONE, kWind3>
+                          : rd_march_kernel<M, ST, 1, ONE, kGeneral>;
+            // batches, whose members differ, keep the general variant
+            const bool windx = ONE && a.windx && !a.plain && !a.wind3;
+            if constexpr (ONE)
+                if (windx) k = rd_march_kernel<M, ST, 1, true, kWindX>;
             threads = LayoutM<M, ST, 1>::threads(a.ty);
-            variant = a.plain ? 4 : a.wind3 ? 5 : 6;
+            variant = a.plain ? 4 : a.wind3 ? 5 : windx ? 7 : 6;
         } else {
             k = rd_step_kernel<M, ST, T, ONE>;
             threads = Layout<M, ST, T>::threads(a.ty);
@@ -907,14 +917,14 @@ cudaError_t launch_one(const LaunchArgs& a, int grid, size_t smem, cudaStream_t 
         if constexpr (T == 2 && !M::CH)
             if (two_step<M, ST>(T, a.ty)) {
                 chained = true;
-                k = a.plain ? rd_march_kernel<M, ST, 2, ONE, true, false>
-                            : rd_march_kernel<M, ST, 2, ONE, false, false>;
+                k = a.plain ? rd_march_kernel<M, ST, 2, ONE, kPlain>
+                            : rd_march_kernel<M, ST, 2, ONE, kGeneral>;
                 threads = LayoutM<M, ST, 2>::threads(a.ty);
                 variant = a.plain ? 1 : 2;
             }
     }
     // dynamic shared memory granted so far, per kernel variant
-    static size_t configured[7] = {0, 0, 0, 0, 0, 0, 0};
+    static size_t configured[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     size_t& conf = configured[variant];
     if (smem > conf) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -29,6 +29,8 @@ def problem(kind, shape):
     src = (nx - 1, 0, nz - 1)                     # on three faces
     if kind == "air":
         return W.air(shape, src=src)
+    if kind == "air_calm":
+        return W.with_(W.air(shape, src=src), wind=None, bc=[[P, P, N, N, P, P]] * 3)
     return W.with_(W.air(shape, src=src), bc=[[N, N, P, P, N, N]] * 3,
                    wind=dict(kind="const", u0=-1.0))
 
@@ -40,7 +42,8 @@ TUNINGS = [dict(tsteps=2, tile_y=8, zchunk=1), dict(tsteps=2, tile_y=12, zchunk=
 
 
 @pytest.mark.parametrize("storage", ["f32", "bf16"])
-@pytest.mark.parametrize("kind", ["diffusion", "turing", "brusselator", "held", "air", "air_mixed"])
+@pytest.mark.parametrize("kind", ["diffusion", "turing", "brusselator", "held", "air", "air_calm",
+                                  "air_mixed"])
 def test_bits_equal_the_multi_level_kernel(kind, storage):
     from paper_1004_0480_gb300.sim import Sim
     for shape in SHAPES:
