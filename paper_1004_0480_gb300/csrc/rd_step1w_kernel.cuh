@@ -182,6 +182,7 @@ rd_step1w_kernel(const __grid_constant__ LaunchArgs a) {
     const int v = tid - r * kQ8;
     const int own_b = ((r + 1) * kRW8 + (v + 1) * kW8) * EB;
 
+    if constexpr (!ONE) chain_wait();   // the batch's counters are read first
     int cur_inst = -1;
     if (tid == 0) s_inst = 0;
     for (long long item = first_item<ONE>(a, s_item); item < a.nitems;
@@ -240,6 +241,7 @@ rd_step1w_kernel(const __grid_constant__ LaunchArgs a) {
         // at a zero-flux x face the neighbour beyond it is the own face cell
         const bool lface = !px && xs == 0;
         const bool rface = !px && xs + kW8 == nx;
+        if constexpr (ONE) chain_wait();   // nothing above reads what a launch writes
         float cy = 0.0f, cz = 0.0f;               // 3-D wind
         if constexpr (W3) wind3d(sd, lin, local, cy, cz);
         __syncthreads();   // halo descriptors written
@@ -368,6 +370,7 @@ rd_step1w_kernel(const __grid_constant__ LaunchArgs a) {
             if (!pz) zq = q + 1;
             else if (++zq == nz) zq = 0;
         }
+        if (ONE && item + gridDim.x >= a.nitems) chain_release();   // the last item
         cp_async_wait<0>();
         __syncthreads();
     }

@@ -877,7 +877,7 @@ cudaError_t launch_one(const LaunchArgs& a, int grid, size_t smem, cudaStream_t 
     int threads = 0;
     // which kernel, and its slot in ``configured`` below
     int variant = 0;
-    bool chained = true;       // march kernels wait for the launch before them
+    bool chained = true;       // the kernels that wait for the launch before them
     if constexpr (T == 1 && M::CH) {
         k = a.plain ? rd_marchch_kernel<M, ST, ONE, true> : rd_marchch_kernel<M, ST, ONE, false>;
         threads = LayoutCH<ST>::threads(a.ty);
@@ -894,7 +894,6 @@ cudaError_t launch_one(const LaunchArgs& a, int grid, size_t smem, cudaStream_t 
                           : rd_step1w_kernel<M, ST, ONE, false, false>;
             threads = Layout1w<M, ST>::threads(a.ty);
             variant = a.plain ? 1 : a.wind3 ? 2 : 3;
-            chained = false;
         } else if (lean) {
             k = a.plain   ? rd_march_kernel<M, ST, 1, ONE, kPlain>
                 : a.wind3 ? rd_march_kernel<M, ST, 1, ONE, kWind3>
