@@ -599,7 +599,7 @@ constexpr double kLaunchUs = 1.9, kPlaneUs = 0.45;
 // What a context steps with while its tuning is the default one: the tile
 // height, z-chunk and steps per launch (at most ``maxT``) of the least
 // modelled cost per step.  Small grids take short chunks (a 97 x 65 x 50
-// Brusselator: 12 rows x 2 planes, 3.0 us a step, where 14 rows x 8 planes
+// Brusselator: 10 rows x 5 planes, 2.7 us a step, where 14 rows x 8 planes
 // at one step per launch took 9.8), large ones the fewest waves; two steps
 // per launch halve the launches and the traffic, but three-species and
 // bfloat16 problems are bound by their arithmetic and keep one where the
@@ -627,14 +627,11 @@ rd_tuning default_plan(const rd_config& g, const rd_tuning& t1, int maxT) {
             };
             const long long cols = (long long)tiles(g.nx, kTileW) * tiles(g.ny, ty);
             const long long slots = (long long)occ * sms;
-            int last = 0;
-            for (int k = 1; k <= g.nz; ++k) {
-                const int zc = tiles(g.nz, k);
-                if (zc == last) continue;
-                last = zc;
+            auto consider = [&](int zc) {
                 const long long items = cols * tiles(g.nz, zc);
                 const long long full = items / slots, rest = items % slots;
-                const double planes = zc + 2 * (T - 1) + 1 + (is_ch(g.model) && sten == 7 ? 2 : 0);
+                const double planes =
+                    zc + 2 * (T - 1) + 1 + (is_ch(g.model) && sten == 7 ? 2 : 0);
                 const double us =
                     planes * (full * plane_us(occ) + plane_us(tiles((int)rest, sms)));
                 const double cost = (kLaunchUs * kernels_per_step(g) + us) / T;
@@ -643,8 +640,18 @@ rd_tuning default_plan(const rd_config& g, const rd_tuning& t1, int maxT) {
                     best = t;
                     best.zchunk = zc;
                 }
-                if (us > 64 * kLaunchUs && zc < 16) break;   // large grid: no shorter chunks
+            };
+            // every split of z that leaves up to four waves of items (at
+            // least 64, at most 1024 splits), and short chunks
+            const long long splits =
+                std::min<long long>({g.nz, 1024, std::max<long long>(64, 4 * slots / cols + 1)});
+            int last = 0;
+            for (int k = 1; k <= splits; ++k) {
+                const int zc = tiles(g.nz, k);
+                if (zc != last) consider(zc);
+                last = zc;
             }
+            for (int zc = std::min(last - 1, 16); zc >= 1; --zc) consider(zc);
         }
     return best;
 }

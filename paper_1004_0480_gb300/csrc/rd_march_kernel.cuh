@@ -304,12 +304,7 @@ struct PlaneFeed {
 enum MarchVar { kGeneral, kPlain, kWind3, kWindX };
 
 template <class M, class ST, int T, bool ONE, int VAR>
-__global__ void
-#ifdef RDM_ATTR
-RDM_ATTR
-#else
-__maxnreg__((LayoutM<M, ST, T>::regs(ONE && VAR == kPlain)))
-#endif
+__global__ void __maxnreg__((LayoutM<M, ST, T>::regs(ONE && VAR == kPlain)))
 rd_march_kernel(const __grid_constant__ LaunchArgs a) {
     static_assert(T == 1 || T == 2, "one or two steps per launch");
     static_assert(VAR != kWindX || T == 1, "the Courant number is read one plane ahead");
