@@ -344,7 +344,6 @@ rd_march_kernel(const __grid_constant__ LaunchArgs a) {
 
     if constexpr (!ONE) chain_wait();   // the batch's counters are read first
     int cur_inst = -1;
-    if (tid == 0) s_inst = 0;
     for (long long item = first_item<ONE>(a, s_item); item < a.nitems;
          item = next_item<ONE>(a, item, s_item)) {
         if constexpr (!ONE) load_desc(a, item, sdm, s_inst, cur_inst);
@@ -562,11 +561,11 @@ rd_march_kernel(const __grid_constant__ LaunchArgs a) {
         };
         for (int e = first;;) {
             body(e, A0, B0, C0, A1, B1, C1);
-            if (++e == z1 + T - 1) break;
+            if (++e >= z1 + T - 1) break;
             body(e, B0, C0, A0, B1, C1, A1);
-            if (++e == z1 + T - 1) break;
+            if (++e >= z1 + T - 1) break;
             body(e, C0, A0, B0, C1, A1, B1);
-            if (++e == z1 + T - 1) break;
+            if (++e >= z1 + T - 1) break;
         }
         if (ONE && item + gridDim.x >= a.nitems) chain_release();   // the last item
         cp_async_wait<0>();

@@ -184,7 +184,6 @@ rd_march19_kernel(const __grid_constant__ LaunchArgs a) {
 
     if constexpr (!ONE) chain_wait();   // the batch's counters are read first
     int cur_inst = -1;
-    if (tid == 0) s_inst = 0;
     for (long long item = first_item<ONE>(a, s_item); item < a.nitems;
          item = next_item<ONE>(a, item, s_item)) {
         if constexpr (!ONE) load_desc(a, item, sdm, s_inst, cur_inst);
@@ -429,11 +428,11 @@ rd_march19_kernel(const __grid_constant__ LaunchArgs a) {
             if constexpr (PASS == 2) lds_vec<ST>(smem + next_slot(slot) + 2 * SPB, DA);
             for (int q = z0;;) {
                 body(q, ZA, ZB, ZC, WA, WB, CA, CB, CC, DA, DB);
-                if (++q == z1) break;
+                if (++q >= z1) break;
                 body(q, ZB, ZC, ZA, WB, WC, CB, CC, CA, DB, DC);
-                if (++q == z1) break;
+                if (++q >= z1) break;
                 body(q, ZC, ZA, ZB, WC, WA, CC, CA, CB, DC, DA);
-                if (++q == z1) break;
+                if (++q >= z1) break;
             }
         } else {   // the halo warp only copies
 #pragma unroll 1

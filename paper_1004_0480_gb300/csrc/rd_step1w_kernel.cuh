@@ -184,7 +184,6 @@ rd_step1w_kernel(const __grid_constant__ LaunchArgs a) {
 
     if constexpr (!ONE) chain_wait();   // the batch's counters are read first
     int cur_inst = -1;
-    if (tid == 0) s_inst = 0;
     for (long long item = first_item<ONE>(a, s_item); item < a.nitems;
          item = next_item<ONE>(a, item, s_item)) {
         if constexpr (!ONE) load_desc(a, item, sdm, s_inst, cur_inst);

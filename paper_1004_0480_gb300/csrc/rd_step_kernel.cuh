@@ -452,7 +452,10 @@ __device__ __forceinline__ const InstDesc& desc_of(const LaunchArgs& a, const In
 }
 
 // Fetch the descriptor of the instance owning ``item`` into ``copy`` (batch
-// launches); one barrier-separated pass per change of instance.
+// launches); one barrier-separated pass per change of instance.  Every item
+// below nitems has exactly one owner, whose thread alone writes s_inst: it
+// needs no initial value, and a store of one by another warp could land after
+// the owner's.
 __device__ __forceinline__ void load_desc(const LaunchArgs& a, long long item, InstDesc& copy,
                                           int& s_inst, int& cur_inst) {
     const int tid = threadIdx.x;
@@ -668,7 +671,6 @@ __global__ void __launch_bounds__(kMaxThreads, 2) rd_step_kernel(const __grid_co
     };
 
     int cur_inst = -1;
-    if (tid == 0) s_inst = 0;
     for (long long item = first_item<ONE>(a, s_item); item < a.nitems;
          item = next_item<ONE>(a, item, s_item)) {
         if constexpr (!ONE) load_desc(a, item, sdm, s_inst, cur_inst);

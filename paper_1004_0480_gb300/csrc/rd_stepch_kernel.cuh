@@ -80,7 +80,6 @@ rd_marchch_kernel(const __grid_constant__ LaunchArgs a) {
 
     if constexpr (!ONE) chain_wait();   // the batch's counters are read first
     int cur_inst = -1;
-    if (tid == 0) s_inst = 0;
     for (long long item = first_item<ONE>(a, s_item); item < a.nitems;
          item = next_item<ONE>(a, item, s_item)) {
         if constexpr (!ONE) load_desc(a, item, sdm, s_inst, cur_inst);
@@ -248,11 +247,11 @@ rd_marchch_kernel(const __grid_constant__ LaunchArgs a) {
         };
         for (int e = first;;) {
             body(e, AA, AB, AC, CA, CB, CC, MA, MB, MX);
-            if (++e == z1 + 1) break;
+            if (++e >= z1 + 1) break;
             body(e, AB, AC, AA, CB, CC, CA, MB, MX, MA);
-            if (++e == z1 + 1) break;
+            if (++e >= z1 + 1) break;
             body(e, AC, AA, AB, CC, CA, CB, MX, MA, MB);
-            if (++e == z1 + 1) break;
+            if (++e >= z1 + 1) break;
         }
         if (ONE && item + gridDim.x >= a.nitems) chain_release();   // the last item
         cp_async_wait<0>();
