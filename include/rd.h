@@ -203,7 +203,10 @@ rd_status rd_create(const rd_config* cfg, rd_ctx** out);
  * (l * nspecies + s) * (state_bytes / (2 * nspecies)); each field is nz
  * planes of ny rows of ``pitch`` elements (float32 or bfloat16), pitch = nx
  * rounded up to a multiple of 128 bytes, x fastest.  Level 0 is current
- * after rd_set_field and after every even number of kernel launches. */
+ * after rd_set_field and after every even number of kernel launches.  Until
+ * a tuning is set (rd_get_tuning then reports one step per launch) a context
+ * on attached memory leaves the levels as one launch per step would: the
+ * current one by the parity of the steps, the step before in the other. */
 rd_status rd_attach(rd_ctx* ctx, void* state, void* scratch);
 
 /* Free what the context owns (device memory, stream, graphs). */

@@ -926,17 +926,23 @@ rd_status step_ctx(rd_ctx* c, int64_t n) {
         c->steps += n;
         return RD_OK;
     }
+    // A caller that attached its own memory reads the levels itself and knows
+    // them by one launch per step, the reported tuning: the plan's two-step
+    // launches then come in an even number with a one-step launch after them,
+    // so the current level has the parity of the steps and the other level
+    // holds the step before.
+    const int64_t pairs = !c->own_mem && c->plan.tsteps == 2 ? (n - 1) / 2 & ~1LL : -1;
     const Use use = c->plan.tsteps == 0 || c->kernel != RD_KERNEL_MARCH ? Use::kTuning
-                    : n >= c->plan.tsteps                               ? Use::kPlan
-                                                                        : Use::kPlan1;
-    if (use == Use::kPlan1 && !c->plan1.tsteps) {   // first call of a single step
+                    : pairs < 0 ? (n >= c->plan.tsteps ? Use::kPlan : Use::kPlan1)
+                                : (pairs ? Use::kPlan : Use::kPlan1);
+    if (use == Use::kPlan1 && !c->plan1.tsteps) {   // first call of single steps
         c->plan1 = default_plan(c->cfg, c->tun, 1);
         fill_desc(c, c->plan1_desc, c->plan1);
     }
     const rd_tuning& t = tuning_of(c, use);
     const int T = t.tsteps;
-    int64_t full = n / T;
-    const int rem = (int)(n % T);
+    int64_t full = use == Use::kPlan && pairs >= 0 ? pairs : n / T;
+    int64_t rem = n - full * T;      // steps after the launches of T
     if (t.graph && full >= kGraphLaunches) {
         st = build_ctx_graph(c, use);
         if (st != RD_OK) return st;
@@ -956,9 +962,11 @@ rd_status step_ctx(rd_ctx* c, int64_t n) {
         if ((st = launch_ctx(c, T, c->cur, c->stream, use)) != RD_OK) return st;
         c->cur ^= 1;
     }
-    if (rem) {
-        if ((st = launch_ctx(c, rem, c->cur, c->stream, use)) != RD_OK) return st;
+    while (rem) {
+        const int k = rem < T ? (int)rem : 1;
+        if ((st = launch_ctx(c, k, c->cur, c->stream, use)) != RD_OK) return st;
         c->cur ^= 1;
+        rem -= k;
     }
     c->steps += n;
     return RD_OK;
