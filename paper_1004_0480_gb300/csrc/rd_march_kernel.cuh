@@ -358,6 +358,7 @@ rd_march_kernel(const __grid_constant__ LaunchArgs a) {
         const int zc = (int)(local / ((long long)sd.ntx * sd.nty));
         const int x0 = txi * kTileQ * kVEC, y0 = tyi * TY;
         const int z0 = zc * sd.zchunk;
+        if (!ONE && z0 >= nz) continue;   // no such item: the march ends on == z1
         const int z1 = min(z0 + sd.zchunk, nz);
         const int lin = sd.par ^ a.parity;
         const ST* const gin = reinterpret_cast<const ST*>(sd.base[lin][0]);
@@ -561,11 +562,11 @@ rd_march_kernel(const __grid_constant__ LaunchArgs a) {
         };
         for (int e = first;;) {
             body(e, A0, B0, C0, A1, B1, C1);
-            if (++e >= z1 + T - 1) break;
+            if (++e == z1 + T - 1) break;
             body(e, B0, C0, A0, B1, C1, A1);
-            if (++e >= z1 + T - 1) break;
+            if (++e == z1 + T - 1) break;
             body(e, C0, A0, B0, C1, A1, B1);
-            if (++e >= z1 + T - 1) break;
+            if (++e == z1 + T - 1) break;
         }
         if (ONE && item + gridDim.x >= a.nitems) chain_release();   // the last item
         cp_async_wait<0>();

@@ -198,6 +198,7 @@ rd_march19_kernel(const __grid_constant__ LaunchArgs a) {
         const int zc = (int)(local / ((long long)sd.ntx * sd.nty));
         const int x0 = txi * kTileQ * kVEC, y0 = tyi * TY;
         const int z0 = zc * sd.zchunk;
+        if (!ONE && z0 >= nz) continue;   // no such item: the march ends on == z1
         const int z1 = min(z0 + sd.zchunk, nz);
         const int lin = sd.par ^ a.parity;
         const ST* const gin = reinterpret_cast<const ST*>(sd.base[lin][PASS == 1 ? 2 : 0]);
@@ -428,11 +429,11 @@ rd_march19_kernel(const __grid_constant__ LaunchArgs a) {
             if constexpr (PASS == 2) lds_vec<ST>(smem + next_slot(slot) + 2 * SPB, DA);
             for (int q = z0;;) {
                 body(q, ZA, ZB, ZC, WA, WB, CA, CB, CC, DA, DB);
-                if (++q >= z1) break;
+                if (++q == z1) break;
                 body(q, ZB, ZC, ZA, WB, WC, CB, CC, CA, DB, DC);
-                if (++q >= z1) break;
+                if (++q == z1) break;
                 body(q, ZC, ZA, ZB, WC, WA, CC, CA, CB, DC, DA);
-                if (++q >= z1) break;
+                if (++q == z1) break;
             }
         } else {   // the halo warp only copies
 #pragma unroll 1

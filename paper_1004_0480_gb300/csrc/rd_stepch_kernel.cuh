@@ -94,6 +94,7 @@ rd_marchch_kernel(const __grid_constant__ LaunchArgs a) {
         const int zc = (int)(local / ((long long)sd.ntx * sd.nty));
         const int x0 = txi * kTileQ * kVEC, y0 = tyi * TY;
         const int z0 = zc * sd.zchunk;
+        if (!ONE && z0 >= nz) continue;   // no such item: the march ends on == z1
         const int z1 = min(z0 + sd.zchunk, nz);
         const int lin = sd.par ^ a.parity;
         const ST* const gin = reinterpret_cast<const ST*>(sd.base[lin][0]);
@@ -247,11 +248,11 @@ rd_marchch_kernel(const __grid_constant__ LaunchArgs a) {
         };
         for (int e = first;;) {
             body(e, AA, AB, AC, CA, CB, CC, MA, MB, MX);
-            if (++e >= z1 + 1) break;
+            if (++e == z1 + 1) break;
             body(e, AB, AC, AA, CB, CC, CA, MB, MX, MA);
-            if (++e >= z1 + 1) break;
+            if (++e == z1 + 1) break;
             body(e, AC, AA, AB, CC, CA, CB, MX, MA, MB);
-            if (++e >= z1 + 1) break;
+            if (++e == z1 + 1) break;
         }
         if (ONE && item + gridDim.x >= a.nitems) chain_release();   // the last item
         cp_async_wait<0>();
