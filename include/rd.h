@@ -179,9 +179,11 @@ rd_status rd_query_sizes(const rd_config* cfg, size_t* state_bytes,
 
 /* Validate ``cfg`` and create a context on the current CUDA device for the
  * problem of eq. (1), discretised by the method of lines (Section 2).
- * Checks: sizes >= 2, species count for the model, periodic faces paired
- * and the same for every species, Dirichlet only on non-periodic faces and
- * not on the Cahn-Hilliard species, and the explicit stability bound
+ * Checks: sizes >= 2, at most 2^34 cells (and planes, with their rows padded
+ * to 128 bytes, of less than 2^34 - 64 elements), species count for the
+ * model, periodic faces paired and the same for every species, Dirichlet only
+ * on non-periodic faces and not on the Cahn-Hilliard species, and the
+ * explicit stability bound
  *   dt * (sum_a 2 D[s][a] / h^2 + |u|max / h) <= 1 for every species
  * (isotropic diffusion: dt <= h^2 / (6 D); the 19-point stencil counts
  * 4 D / h^2 instead), plus, for the Cahn-Hilliard species,

@@ -315,6 +315,12 @@ int periodic_axis(const rd_config& c, int s, int a) {
     return c.bc[s][2 * a] == RD_BC_PERIODIC;
 }
 
+// elements per row: rows padded to 128 bytes so 16-byte vectors never cross a
+// row end
+int pitch_of(const rd_config& g) {
+    return (int)align_up((size_t)g.nx, (size_t)(128 / elem_bytes(g.storage)));
+}
+
 rd_status validate(const rd_config* c) {
     if (!c) return fail(nullptr, RD_EINVAL, "null config");
     if (c->nx < 2 || c->ny < 2 || c->nz < 2)
@@ -340,6 +346,8 @@ rd_status validate(const rd_config* c) {
     }
     if (c->storage != RD_STORE_F32 && c->storage != RD_STORE_BF16)
         return fail(nullptr, RD_EINVAL, "unknown storage %d", c->storage);
+    if (!plane_fits((long long)pitch_of(*c) * c->ny))
+        return fail(nullptr, RD_EINVAL, "grid too large: a plane of %d padded rows", c->ny);
     for (int s = 0; s < c->nspecies; ++s) {
         for (int f = 0; f < 6; ++f)
             if (c->bc[s][f] < RD_BC_NEUMANN || c->bc[s][f] > RD_BC_DIRICHLET)
@@ -446,9 +454,7 @@ void layout(rd_ctx* c) {
     c->S = g.nspecies;
     c->vec = vec_of(g.storage);
     c->ebytes = elem_bytes(g.storage);
-    // rows padded to 128 bytes so 16-byte vectors never cross a row end
-    const int row_align = 128 / c->ebytes;
-    c->pitch = (int)align_up((size_t)g.nx, (size_t)row_align);
+    c->pitch = pitch_of(g);
     c->plane = (long long)c->pitch * g.ny;
     c->field_bytes = align_up((size_t)c->plane * g.nz * c->ebytes, 256);
     c->state_bytes = c->field_bytes * 2 * c->S;

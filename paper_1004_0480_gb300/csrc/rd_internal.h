@@ -13,6 +13,14 @@ constexpr int kMaxThreads = 512;     // upper bound of step-kernel CTA size
 constexpr int kTileQ = 16;           // tile width in 4-cell vectors (64 cells)
 constexpr int kMaxS = RD_MAX_SPECIES;
 
+// The step kernels' copy offsets within a plane count 4-cell vectors (rows are
+// whole vectors) in 32 unsigned bits, so that no 64-bit value is kept per
+// fetch; cell offsets would leave an int beyond 2^31 cells.  rd_create refuses
+// planes past the limit, 2^34 cells but for a few vectors (two values are
+// codes of the 19-point kernel): only rows of at most 32 cells, padded to 128
+// bytes, reach it within the accepted cell counts.
+inline bool plane_fits(long long plane) { return plane / 4 < 0xfffffff0LL; }
+
 // One instance (context) as the step kernels see it.  Written by the host,
 // read by every CTA that works on the instance.
 struct InstDesc {

@@ -129,9 +129,14 @@ template <class M, class ST, int T> struct LayoutM {
 
 // Mirror extension: -1-i for i < 0, 2n-1-i for i >= n; clamped so that
 // positions outside the grid by more than n (never stored) stay in bounds.
-__device__ __forceinline__ int mirror_index(int i, int n) {
+__host__ __device__ __forceinline__ int mirror_index(int i, int n) {
     const int m = i < 0 ? -1 - i : (i >= n ? 2 * n - 1 - i : i);
     return min(max(m, 0), n - 1);
+}
+
+// Offset of the row that stands for row ``yrow`` within a plane, in vectors.
+__host__ __device__ __forceinline__ unsigned row_offset(int yrow, int ny, int pitch, bool py) {
+    return (unsigned)(py ? wrapi(yrow, ny) : mirror_index(yrow, ny)) * ((unsigned)pitch / kVEC);
 }
 
 // How one vector of a march is fetched: rows beyond a zero-flux y face are
@@ -139,21 +144,21 @@ __device__ __forceinline__ int mirror_index(int i, int n) {
 // face are not fetched, and the last vector of a row that ends inside it is
 // copied whole (its tail is the row's padding, never read).
 template <class ST>
-__device__ __forceinline__ Fetch make_fetch_h(int yrow, int xs, int nx, int ny, int pitch, bool px,
-                                             bool py, int soff_bytes) {
+__host__ __device__ __forceinline__ Fetch make_fetch_h(int yrow, int xs, int nx, int ny, int pitch,
+                                                      bool px, bool py, int soff_bytes) {
     Fetch f{0, 0, soff_bytes, xs};
     if (yrow > ny + 1 || xs > nx + 1) return f;          // feeds no stored cell
-    const int row = (py ? wrapi(yrow, ny) : mirror_index(yrow, ny)) * pitch;
+    const unsigned row = row_offset(yrow, ny, pitch, py);
     if (xs >= 0 && xs + kVEC <= nx) {
         f.mode = 1;
-        f.goff = row + xs;
+        f.goff = row + (unsigned)xs / kVEC;
     } else if (px) {
         const int xw = wrapi(xs, nx);
-        if (xw % kVEC == 0 && xw + kVEC <= nx) { f.mode = 1; f.goff = row + xw; }
+        if (xw % kVEC == 0 && xw + kVEC <= nx) { f.mode = 1; f.goff = row + (unsigned)xw / kVEC; }
         else { f.mode = 2; f.goff = row; }
     } else if (xs >= 0 && xs < nx) {
         f.mode = 1;
-        f.goff = row + xs;
+        f.goff = row + (unsigned)xs / kVEC;
     }
     return f;
 }
@@ -169,7 +174,7 @@ __device__ __forceinline__ void fetch_elems(const Fetch& f, unsigned char* dst, 
         ST* d = reinterpret_cast<ST*>(dst + s * pe_bytes + f.soff);
 #pragma unroll
         for (int e = 0; e < kVEC; ++e) {
-            const ST* src = gplane + s * fstride + f.goff + wrapi(f.xs + e, nx);
+            const ST* src = vec_at(gplane, f.goff) + s * fstride + wrapi(f.xs + e, nx);
             if (RD_DBG_GLOBAL(sd, src, (int)sizeof(ST), kSiteCopySrc))
                 Store<ST>::cp_async_elem(d + e, src);
         }
@@ -414,7 +419,7 @@ rd_march_kernel(const __grid_constant__ LaunchArgs a) {
                     if (k == 0 || !inner_warp)   // (no break: f stays in registers)
 #pragma unroll
                     for (int s = 0; s < S; ++s) {
-                        const ST* gs = g + f[k].goff + s * fstride;
+                        const ST* gs = vec_at(g, f[k].goff) + s * fstride;
                         const int ok = f[k].mode == 1 &&
                                        RD_DBG_GLOBAL(sd, gs, 4 * (int)sizeof(ST), kSiteCopySrc);
                         Store<ST>::cp_async_if(

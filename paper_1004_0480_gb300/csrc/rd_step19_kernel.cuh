@@ -226,13 +226,14 @@ rd_march19_kernel(const __grid_constant__ LaunchArgs a) {
         if constexpr (ONE) chain_wait();   // nothing above reads what a launch writes
         float cy = 0.0f, cz = 0.0f;                   // 3-D wind
         if constexpr (W3 && PASS == 0) wind3d(sd, lin, local, cy, cz);
-        // what the thread copies of every plane: its own vector, element
-        // offset ``go`` of a plane (-1: none, -2: element by element), or for
-        // the halo warp three vectors a lane, described in shared memory
-        int go = -1;
+        // what the thread copies of every plane: its own vector, offset ``go``
+        // of a plane (kNone: none, kElems: element by element), or for the halo
+        // warp three vectors a lane, described in shared memory
+        constexpr unsigned kNone = 0xffffffffu, kElems = 0xfffffffeu;
+        unsigned go = kNone;
         if (inner) {
             const Fetch f = make_fetch_h<ST>(y, xs, nx, ny, pitch, px, py, 0);
-            go = f.mode == 1 ? f.goff : -f.mode;
+            go = f.mode == 1 ? f.goff : f.mode == 2 ? kElems : 0;
         } else {
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
@@ -242,7 +243,7 @@ rd_march19_kernel(const __grid_constant__ LaunchArgs a) {
                                                  pitch, px, py,
                                                  kGuard19 + h.r * ROWB + h.v * kVEC * EB);
                 if (RD_DBG_SHARED(hfetch + hl + 32 * k, 16, kSiteHaloDesc))
-                    hfetch[hl + 32 * k] = make_int4(f.mode, f.goff, f.soff, f.xs);
+                    hfetch[hl + 32 * k] = make_int4(f.mode, (int)f.goff, f.soff, f.xs);
             }
             __syncwarp();
         }
@@ -253,16 +254,17 @@ rd_march19_kernel(const __grid_constant__ LaunchArgs a) {
         PlaneFeed feed(z0 - 1, nz, pz);
         const int slot_end = own0 + RING * SLOTB;
         int slot_ld = own0;
-        // the vector at element offset o of the plane at goff, to d (mu: dm)
-        auto copy = [&](long long goff, int o, unsigned char* d, unsigned char* dm, bool ok) {
-            const ST* const g = gin + goff + o;
+        // vector o of the plane at goff, to d (mu: dm)
+        auto copy = [&](long long goff, unsigned o, unsigned char* d, unsigned char* dm, bool ok) {
+            goff += (unsigned long long)o * kVEC;
+            const ST* const g = gin + goff;
 #pragma unroll
             for (int s = 0; s < NS; ++s)
                 Store<ST>::cp_async_if(
                     reinterpret_cast<ST*>(d + s * SPB), g + s * fstride,
                     ok && RD_DBG_GLOBAL(sd, g + s * fstride, 4 * (int)sizeof(ST), kSiteCopySrc));
             if constexpr (MUF) {
-                const float* const gm = sd.mu + goff + o;
+                const float* const gm = sd.mu + goff;
                 Store<float>::cp_async_if(reinterpret_cast<float*>(dm), gm,
                                           ok && RD_DBG_GLOBAL(sd, gm, 16, kSiteMu));
             }
@@ -279,22 +281,22 @@ rd_march19_kernel(const __grid_constant__ LaunchArgs a) {
                 const long long goff = (long long)feed.plane() * plane;
                 unsigned char* const d = smem + slot_ld;
                 if (inner_warp) {
-                    copy(goff, go, d, d + mu_own, go >= 0);
+                    copy(goff, go, d, d + mu_own, go < kElems);
                 } else {
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
                         const int4 h = hfetch[hl + 32 * k];
                         unsigned char* const dk = d - own0 + h.z;
-                        copy(goff, h.y, dk, dk + mu_shift(h.w), h.x == 1);
+                        copy(goff, (unsigned)h.y, dk, dk + mu_shift(h.w), h.x == 1);
                     }
                 }
                 if (elems) {   // periodic x, nx not a multiple of 4
-                    if (go == -2)
-                        copy_elems(goff, make_fetch_h<ST>(y, xs, nx, ny, pitch, px, py, 0), d);
+                    if (go == kElems)
+                        copy_elems(goff, Fetch{2, row_offset(y, ny, pitch, py), 0, xs}, d);
                     if (!inner_warp)
                         for (int k = 0; k < 3; ++k) {
                             const int4 h = hfetch[hl + 32 * k];
-                            copy_elems(goff, Fetch{h.x, h.y, h.z, h.w}, d - own0);
+                            copy_elems(goff, Fetch{h.x, (unsigned)h.y, h.z, h.w}, d - own0);
                         }
                 }
             }

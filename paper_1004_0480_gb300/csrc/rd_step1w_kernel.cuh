@@ -89,19 +89,19 @@ template <> struct Vec8<__nv_bfloat16> {
 // How one 8-cell vector is fetched: rows beyond a zero-flux face are the face
 // row, cells beyond one in x clamped.
 template <class ST>
-__device__ __forceinline__ Fetch make_fetch8(int yrow, int xs, int nx, int ny, int pitch, bool px,
-                                             bool py, int soff_elems) {
+__host__ __device__ __forceinline__ Fetch make_fetch8(int yrow, int xs, int nx, int ny, int pitch,
+                                                     bool px, bool py, int soff_elems) {
     Fetch f{0, 0, soff_elems * (int)sizeof(ST), xs};
     int yw = yrow;
     if (py) yw = wrapi(yrow, ny);
     else if (yrow < 0 || yrow >= ny) yw = yrow < 0 ? 0 : ny - 1;    // ghost row = face row
-    const int row = yw * pitch;
+    const unsigned row = (unsigned)yw * ((unsigned)pitch / kVEC);
     if (xs >= 0 && xs + kW8 <= nx) {
         f.mode = 1;
-        f.goff = row + xs;
+        f.goff = row + (unsigned)xs / kVEC;
     } else if (px) {
         const int xw = wrapi(xs, nx);
-        if (xw % kW8 == 0 && xw + kW8 <= nx) { f.mode = 1; f.goff = row + xw; }
+        if (xw % kW8 == 0 && xw + kW8 <= nx) { f.mode = 1; f.goff = row + (unsigned)xw / kVEC; }
         else { f.mode = 2; f.goff = row; }
     } else if (xs < nx && xs + kW8 > 0) {
         f.mode = 2;                               // straddles a face: clamped ghosts
@@ -116,7 +116,7 @@ __device__ __forceinline__ void fetch_all8(const Fetch& f, unsigned char* plane_
                                            const InstDesc& sd) {
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-        const ST* src = gplane + s * fstride + f.goff;
+        const ST* src = vec_at(gplane, f.goff) + s * fstride;
         const int ok =
             f.mode == 1 && RD_DBG_GLOBAL(sd, src, kW8 * (int)sizeof(ST), kSiteCopySrc);
         Vec8<ST>::cp_async_if(reinterpret_cast<ST*>(plane_buf + s * pe_bytes + f.soff), src, ok);
@@ -129,7 +129,7 @@ __device__ __forceinline__ void fetch_all8(const Fetch& f, unsigned char* plane_
             for (int e = 0; e < kW8; ++e) {
                 const int x = f.xs + e;
                 const int xi = px ? wrapi(x, nx) : (x < 0 ? 0 : (x >= nx ? nx - 1 : x));
-                const ST* src = gplane + s * fstride + f.goff + xi;
+                const ST* src = vec_at(gplane, f.goff) + s * fstride + xi;
                 if (RD_DBG_GLOBAL(sd, src, (int)sizeof(ST), kSiteCopySrc))
                     Store<ST>::cp_async_elem(d + e, src);
             }
@@ -226,7 +226,7 @@ rd_step1w_kernel(const __grid_constant__ LaunchArgs a) {
                                         px, py, (bottom ? TY + 1 : 0) * kRW8 + (hv + 1) * kW8);
                 }
                 if (RD_DBG_SHARED(hfetch + j, 16, kSiteHaloDesc))
-                    hfetch[j] = make_int4(f.mode, f.goff, f.soff, f.xs);
+                    hfetch[j] = make_int4(f.mode, (int)f.goff, f.soff, f.xs);
             }
         }
         // ---- compute threads: own vector and its neighbours
@@ -261,8 +261,8 @@ rd_step1w_kernel(const __grid_constant__ LaunchArgs a) {
                         int4 h = make_int4(0, 0, 0, 0);
                         if (RD_DBG_SHARED(hfetch + hl + 32 * k, 16, kSiteHaloDesc))
                             h = hfetch[hl + 32 * k];
-                        fetch_all8<ST, S>(Fetch{h.x, h.y, h.z, h.w}, buf, PEB, gld, fstride, nx,
-                                          px, sd);
+                        fetch_all8<ST, S>(Fetch{h.x, (unsigned)h.y, h.z, h.w}, buf, PEB, gld,
+                                          fstride, nx, px, sd);
                     }
                 } else {
                     fetch_all8<ST, S>(fo, buf, PEB, gld, fstride, nx, px, sd);

@@ -149,7 +149,7 @@ template <int N> __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
-__device__ __forceinline__ int wrapi(int i, int n) {
+__host__ __device__ __forceinline__ int wrapi(int i, int n) {
     int r = i % n;
     return r < 0 ? r + n : r;
 }
@@ -844,10 +844,16 @@ __global__ void __launch_bounds__(kMaxThreads, 2) rd_step_kernel(const __grid_co
 // straddling a zero-flux face), 0 = nothing.
 struct Fetch {
     int mode;
-    int goff;    // element offset of row + x within a plane
+    unsigned goff;   // offset of row + x (mode 2: of the row) within a plane, in
+                     // 4-cell vectors (plane_fits, rd_internal.h)
     int soff;    // byte offset of the position within a plane buffer
     int xs;      // global x of the vector's first element (unwrapped)
 };
+
+// the 4-cell vector ``v`` vectors past p
+template <class ST> __host__ __device__ __forceinline__ const ST* vec_at(const ST* p, unsigned v) {
+    return p + (unsigned long long)v * kVEC;
+}
 
 template <class ST>
 __device__ __forceinline__ void lds_vec(const unsigned char* p, float (&v)[kVEC]) {

@@ -127,13 +127,13 @@ rd_marchch_kernel(const __grid_constant__ LaunchArgs a) {
                 unsigned char* const d = smem + slot_ld;
 #pragma unroll
                 for (int s = 0; s < S; ++s) {
-                    const ST* gs = g + fo.goff + s * fstride;
+                    const ST* gs = vec_at(g, fo.goff) + s * fstride;
                     const int ok = fo.mode == 1 &&
                                    RD_DBG_GLOBAL(sd, gs, 4 * (int)sizeof(ST), kSiteCopySrc);
                     Store<ST>::cp_async_if(reinterpret_cast<ST*>(d + s * RM::SPB), gs, ok);
                 }
                 if (halo_warp) {
-                    const ST* gs = g + fx.goff + 2 * fstride;
+                    const ST* gs = vec_at(g, fx.goff) + 2 * fstride;
                     const int ok = fx.mode == 1 &&
                                    RD_DBG_GLOBAL(sd, gs, 4 * (int)sizeof(ST), kSiteCopySrc);
                     Store<ST>::cp_async_if(reinterpret_cast<ST*>(d + fx.soff), gs, ok);
