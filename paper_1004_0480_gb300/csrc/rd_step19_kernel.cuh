@@ -74,6 +74,14 @@ template <class M, class ST, int PASS> struct Layout19 {
     __host__ __device__ static int threads(int ty) { return kTileQ * ty + 32; }
 };
 
+// A fetch of the own vector in one word: its offset, or kNone (positions
+// outside the grid, in tiles that it does not fill, copy nothing) or kElems
+// (element by element).
+constexpr unsigned kNone = 0xffffffffu, kElems = 0xfffffffeu;
+__host__ __device__ __forceinline__ unsigned own_offset(const Fetch& f) {
+    return f.mode == 1 ? f.goff : f.mode == 2 ? kElems : kNone;
+}
+
 // Own vector c and the sums Z, W of one field's plane at the thread's 4
 // cells; ``p`` points at the own vector in the ring, rows ROWB bytes apart.
 // The x neighbours of a pair are no aligned pair of registers: sums along x
@@ -227,13 +235,12 @@ rd_march19_kernel(const __grid_constant__ LaunchArgs a) {
         float cy = 0.0f, cz = 0.0f;                   // 3-D wind
         if constexpr (W3 && PASS == 0) wind3d(sd, lin, local, cy, cz);
         // what the thread copies of every plane: its own vector, offset ``go``
-        // of a plane (kNone: none, kElems: element by element), or for the halo
-        // warp three vectors a lane, described in shared memory
-        constexpr unsigned kNone = 0xffffffffu, kElems = 0xfffffffeu;
+        // of a plane (see own_offset), or for the halo warp three vectors a
+        // lane, described in shared memory
         unsigned go = kNone;
         if (inner) {
             const Fetch f = make_fetch_h<ST>(y, xs, nx, ny, pitch, px, py, 0);
-            go = f.mode == 1 ? f.goff : f.mode == 2 ? kElems : 0;
+            go = own_offset(f);
         } else {
 #pragma unroll
             for (int k = 0; k < 3; ++k) {

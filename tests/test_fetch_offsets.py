@@ -1,10 +1,10 @@
 """Where the step kernels copy from: the offset of every fetch within a plane,
 on the host, against 64-bit arithmetic.  Planes of 2^31 cells and more (two
 such planes are within the accepted 2^34 cells) must not overflow, planes past
-the offsets' range are refused, and the
-smallest and odd planes keep their rules: wrapped rows and columns on periodic
-axes, mirrored (march kernels) or clamped (8-cell kernel) rows beyond
-zero-flux faces."""
+the offsets' range are refused, and the smallest and odd planes keep their
+rules: wrapped rows and columns on periodic axes, mirrored (march kernels) or
+clamped (8-cell kernel) rows beyond zero-flux faces, nothing where no stored
+cell needs a vector."""
 import ctypes
 import shutil
 import subprocess
@@ -17,7 +17,7 @@ from paper_1004_0480_gb300 import workloads as W
 
 PROGRAM = r"""
 #include <cstdio>
-#include "rd_step_kernel.cuh"
+#include "rd_step19_kernel.cuh"
 using namespace rdk;
 typedef long long ll;
 
@@ -31,9 +31,9 @@ static void check(const char* what, const Fetch& f, int w, ll row, int xs, int n
     // no single copy: wraps round, straddles a face (8-cell kernel)
     const bool split = px ? x % w || x + w > nx : w == kW8 && x + w > nx;
     bool ok;
-    if (none) ok = f.mode == 0;
-    else if (split) ok = f.mode == 2 && (ll)f.goff * kVEC == row * pitch && f.xs == xs;
-    else ok = f.mode == 1 && (ll)f.goff * kVEC == row * pitch + x && x + w <= pitch;
+    if (none) ok = f.mode == 0 && own_offset(f) == kNone;   // not the plane's first vector
+    else if (split) ok = f.mode == 2 && own_offset(f) == kElems && (ll)f.goff * kVEC == row * pitch && f.xs == xs;
+    else ok = f.mode == 1 && own_offset(f) == f.goff && (ll)f.goff * kVEC == row * pitch + x && x + w <= pitch;
     if (!ok && bad++ < 5)
         std::printf("%s: row %lld of pitch %lld, x %d of %d: mode %d, offset %u\n", what, row,
                     pitch, xs, nx, f.mode, f.goff);
