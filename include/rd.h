@@ -222,7 +222,8 @@ rd_status rd_set_stream(rd_ctx* ctx, void* stream);
  * into species ``s`` of the current level, converting to the storage type
  * (the host loop's copy of the initial state to the GPU, Table 3).
  * Cells of held (Dirichlet) layers are set to their bc_value.  Returns
- * after the source buffer may be reused. */
+ * after the source buffer may be reused.  RD_EINVAL for device memory that
+ * ends before ``count`` values (here and in rd_get_field). */
 rd_status rd_set_field(rd_ctx* ctx, int s, const float* src, size_t count);
 
 /* Advance every species by ``nsteps`` forward-Euler steps (eq. (5)).

@@ -23,6 +23,7 @@
 #include "rd.h"
 #include "rd_internal.h"
 #include "rd_ablation.h"
+#include "rd_extent.h"
 #include "rd_model_turing.h"
 #include "rd_resident.h"
 #include "rd_step19.h"
@@ -992,23 +993,46 @@ bool is_device_ptr(const void* p) {
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-// Whether the pack and unpack kernels may read or write the caller's ``n``
-// floats at p themselves: device memory of the current device, aligned, apart
-// from the context's own memory.  Anything else goes through the staging
-// field.
-bool kernel_may_touch(const rd_ctx* c, const void* p, size_t n) {
+// cuMemGetAddressRange from the driver, found once through the runtime (no
+// link against the driver library); null when unavailable.
+using RangeFn = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+RangeFn range_fn() {
+    static const RangeFn fn = []() -> RangeFn {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault,
+                                             &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            return nullptr;
+        return reinterpret_cast<RangeFn>(f);
+    }();
+    return fn;
+}
+
+// How the caller's ``n`` floats at p reach the context's field: kDirect, the
+// pack and unpack kernels read or write them themselves (device memory of the
+// current device, one allocation, aligned, apart from the context's own
+// memory); kShort, refused, since the memory ends before them and nothing
+// would stop a kernel; kStaged, anything else, by a copy to the staging field
+// that the runtime checks.
+enum class Route { kDirect, kStaged, kShort };
+Route field_route(const rd_ctx* c, const void* p, size_t n) {
     cudaPointerAttributes at{};
     int dev = -1;
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return Route::kStaged;
     }
-    if (at.type != cudaMemoryTypeDevice || at.device != dev) return false;
+    if (at.type != cudaMemoryTypeDevice || at.device != dev || !range_fn()) return Route::kStaged;
     const char* lo = static_cast<const char*>(p);
     const char* hi = lo + n * sizeof(float);
-    if (reinterpret_cast<uintptr_t>(p) % sizeof(float)) return false;
+    const Extent ext = extent_of(range_fn(), reinterpret_cast<CUdeviceptr>(p), n * sizeof(float));
+    if (ext == Extent::kShort) return Route::kShort;
+    if (ext != Extent::kOne || reinterpret_cast<uintptr_t>(p) % sizeof(float))
+        return Route::kStaged;
     auto apart = [&](const char* m, size_t bytes) { return hi <= m || lo >= m + bytes; };
-    return apart(c->state, c->state_bytes) && apart(c->scratch, c->scratch_bytes);
+    return apart(c->state, c->state_bytes) && apart(c->scratch, c->scratch_bytes) ? Route::kDirect
+                                                                                 : Route::kStaged;
 }
 
 std::mutex g_tune_mu;
@@ -1158,7 +1182,10 @@ rd_status rd_set_field(rd_ctx* c, int s, const float* src, size_t count) {
     const rd_config& g = c->cfg;
     const size_t n = (size_t)g.nx * g.ny * g.nz;
     if (count != n) return fail(c, RD_EINVAL, "count %zu != nx*ny*nz = %zu", count, n);
-    const bool direct = kernel_may_touch(c, src, n);
+    const Route route = field_route(c, src, n);
+    if (route == Route::kShort)
+        return fail(c, RD_EINVAL, "the buffer's memory ends before its %zu values", n);
+    const bool direct = route == Route::kDirect;
     if (!direct)
         RD_CUDA(c, cudaMemcpyAsync(c->staging, src, n * sizeof(float),
                                    is_device_ptr(src) ? cudaMemcpyDeviceToDevice
@@ -1186,7 +1213,10 @@ rd_status rd_get_field(rd_ctx* c, int s, float* dst, size_t count) {
     const rd_config& g = c->cfg;
     const size_t n = (size_t)g.nx * g.ny * g.nz;
     if (count != n) return fail(c, RD_EINVAL, "count %zu != nx*ny*nz = %zu", count, n);
-    const bool direct = kernel_may_touch(c, dst, n);
+    const Route route = field_route(c, dst, n);
+    if (route == Route::kShort)
+        return fail(c, RD_EINVAL, "the buffer's memory ends before its %zu values", n);
+    const bool direct = route == Route::kDirect;
     cudaError_t e = launch_unpack(field_ptr(c, c->cur, s), direct ? dst : c->staging, g.storage,
                                   g.nx, g.ny, g.nz, c->pitch, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "unpack kernel");

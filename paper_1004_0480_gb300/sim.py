@@ -160,8 +160,11 @@ class Sim:
         if out is None:
             out = np.empty((nz, ny, nx), dtype=np.float32)
         addr, keep = _ptr(out)
-        self._check(self.lib.rd_get_field(self.ctx, s, ctypes.c_void_p(addr), self.ncell),
-                    "rd_get_field")
+        n = self.ncell
+        count = keep.size if isinstance(keep, np.ndarray) else keep.numel()
+        if count < n:
+            raise ValueError(f"out has room for {count} values, the grid has {n}")
+        self._check(self.lib.rd_get_field(self.ctx, s, ctypes.c_void_p(addr), n), "rd_get_field")
         return out
 
     def get_fields(self):
