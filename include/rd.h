@@ -492,6 +492,12 @@ rd_status rd_batch_sync(rd_batch* b);
 rd_status rd_batch_destroy(rd_batch* b);
 int64_t rd_batch_launch_count(const rd_batch* b);
 
+/* Testing hook (the paper has no counterpart): out[0] = CTAs of the batch's
+ * last step launch, out[1] = CTAs of that kernel that the GPU holds at once.
+ * RD_EINVAL for a null argument or before the first launch of two or more
+ * members. */
+rd_status rd_debug_batch_grid(const rd_batch* b, int64_t out[2]);
+
 #ifdef __cplusplus
 }
 #endif

@@ -199,17 +199,20 @@ int variant_code(const rd_config& g) {
     return plain_problem(g) ? 1 : g.wind_kind == RD_WIND_3D ? 2 : windx_problem(g) ? 3 : 0;
 }
 
+// ``batch``: of the form that batches launch, whose register budgets differ
+// (LayoutM::regs): a plain 14-row diffusion kernel fits 4 CTAs on an SM alone
+// and 3 in a batch, a two-species one 3 and 2.
 int occupancy(int model, int storage, int T, int ty, int regcap = 0, int plain = 0,
-              int stencil = 7, int tq = kTileQ) {
+              int stencil = 7, int tq = kTileQ, bool batch = false) {
     static std::mutex mu;
-    static std::map<std::tuple<int, int, int, int, int, int, int, int>, int> cache;
+    static std::map<std::tuple<int, int, int, int, int, int, int, int, bool>, int> cache;
     std::lock_guard<std::mutex> g(mu);
-    auto key = std::make_tuple(model, storage, T, ty, regcap, plain, stencil, tq);
+    auto key = std::make_tuple(model, storage, T, ty, regcap, plain, stencil, tq, batch);
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;
     int occ = 0;
     LaunchArgs dummy{};
-    dummy.use_one = 1;
+    dummy.use_one = !batch;
     dummy.regcap = regcap;
     // plain: a variant_code
     dummy.plain = plain == 1;
@@ -287,6 +290,11 @@ struct rd_batch {
     Graph graph;
     long long members_version = 0;
     int64_t launches = 0;
+    // the last step launch (rd_debug_batch_grid)
+    LaunchArgs last{};
+    int last_T = 0;
+    long long last_grid = 0;
+    size_t last_smem = 0;
 };
 
 namespace {
@@ -1653,6 +1661,17 @@ rd_status rd_batch_set_tuning(rd_batch* b, const rd_tuning* t) {
 
 namespace {
 
+// the kernel variant that a batch's members share (as variant_code; batches
+// have no kernel of their own for the wind along x)
+int batch_variant(const rd_batch* b) {
+    bool plain = true, wind3 = false;
+    for (const rd_ctx* m : b->members) {
+        plain = plain && plain_problem(m->cfg);
+        wind3 = wind3 || m->cfg.wind_kind == RD_WIND_3D;
+    }
+    return plain ? 1 : wind3 ? 2 : 0;
+}
+
 // The batch's tuning: the one set by rd_batch_set_tuning, else one step per
 // launch at the default tile height with a z-chunk that fills the CTA slots
 // over all current members.
@@ -1663,7 +1682,8 @@ rd_tuning batch_tuning(rd_batch* b) {
     t.tile_q = kTileQ;
     t.tile_y = default_tile_y(b->model);
     t.graph = 1;
-    const int occ = occupancy(b->model, b->storage, 1, t.tile_y, 0, 0, b->stencil);
+    const int occ = occupancy(b->model, b->storage, 1, t.tile_y, 0, batch_variant(b), b->stencil,
+                              kTileQ, true);
     std::vector<std::pair<long long, int>> cols_nz;
     for (rd_ctx* c : b->members)
         cols_nz.push_back({(long long)tiles(c->cfg.nx, kTileW) *
@@ -1750,18 +1770,19 @@ rd_status batch_launch(rd_batch* b, const rd_tuning& t, int T, int parity, long 
     a.parity = parity;
     a.nitems = nitems;
     a.regcap = t.regcap;
-    a.plain = 1;
-    for (rd_ctx* m : b->members) {
-        a.plain = a.plain && plain_problem(m->cfg);
-        a.wind3 = a.wind3 || m->cfg.wind_kind == RD_WIND_3D;
-    }
+    const int variant = batch_variant(b);
+    a.plain = variant == 1;
+    a.wind3 = variant == 2;
     a.ty = t.tile_y;
     a.vw = vw_of(t.tile_q);
     const size_t sm = smem_of(b->model, b->storage, T, a.ty, b->stencil, t.tile_q);
     const int occ = std::max(
-        1, occupancy(b->model, b->storage, T, a.ty, a.regcap, a.plain ? 1 : a.wind3 ? 2 : 0,
-                     b->stencil, t.tile_q));
+        1, occupancy(b->model, b->storage, T, a.ty, a.regcap, variant, b->stencil, t.tile_q, true));
     const long long grid = std::min<long long>(nitems, (long long)occ * num_sms());
+    b->last = a;
+    b->last_T = T;
+    b->last_grid = grid;
+    b->last_smem = sm;
     a.work = (caps || nitems >= 4 * grid) ? b->work : nullptr;
     cudaError_t e = launch_model(b->model, b->storage, T, a, (int)grid, sm, st, nullptr, b->stencil);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch step launch");
@@ -1902,5 +1923,17 @@ rd_status rd_batch_destroy(rd_batch* b) {
 }
 
 int64_t rd_batch_launch_count(const rd_batch* b) { return b ? b->launches : -1; }
+
+rd_status rd_debug_batch_grid(const rd_batch* b, int64_t out[2]) {
+    if (!b || !out) return fail(nullptr, RD_EINVAL, "null argument");
+    if (!b->last_T) return fail(nullptr, RD_EINVAL, "the batch has launched nothing");
+    int occ = 0;
+    const cudaError_t e = launch_model(b->model, b->storage, b->last_T, b->last, 0, b->last_smem,
+                                       nullptr, &occ, b->stencil);
+    if (e != cudaSuccess) return cuda_fail(nullptr, e, "occupancy");
+    out[0] = b->last_grid;
+    out[1] = (int64_t)occ * num_sms();
+    return RD_OK;
+}
 
 }  // extern "C"

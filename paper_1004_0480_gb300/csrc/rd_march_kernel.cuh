@@ -108,7 +108,7 @@ template <class M, class ST, int T> struct LayoutM {
     //   the same in BF16, T = 2: 441 (128) 362 (112) 312 (96)
     //                     T = 1: 457 (128) 451 (96) 401 (80) 296 (64)
     //   air 512 x 512 x 64 FP32, T = 1: 253 (128) 249 (112) 215 (96)
-    // The general and batch variants take 16 more.
+    // The general variants and batches take 16 more where that is below 128.
     static constexpr int regs(bool lean) {
         if (S == 3 || (S == 2 && sizeof(ST) == 2)) return 128;
         return (S == 2 ? (T == 2 ? 96 : 80) : (T == 2 ? 80 : 64)) + (lean ? 0 : 16);

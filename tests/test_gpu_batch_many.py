@@ -61,3 +61,37 @@ def test_many_members_equal_their_own_runs(model, stencil, storage):
     for t in TUNINGS["ch" if model == "ch_front" and stencil == 7 else stencil]:
         for i, (a, b) in enumerate(zip(run(t), ref)):
             assert np.array_equal(a.view(np.uint32), b.view(np.uint32)), (t, cfgs[i]["shape"])
+
+
+@pytest.mark.parametrize("model,stencil,storage", [
+    ("diffusion", 7, "f32"), ("diffusion", 7, "bf16"), ("brusselator", 7, "f32"),
+    ("brusselator", 7, "bf16"), ("air", 7, "f32"), ("ch_front", 7, "f32"),
+    ("diffusion", 19, "f32"), ("brusselator", 19, "f32")])
+@pytest.mark.parametrize("tsteps", [1, 2])
+def test_a_batch_launches_the_ctas_that_fit(model, stencil, storage, tsteps):
+    """A persistent batch kernel with more CTAs than the GPU holds starts the
+    surplus after the others have taken their whole lists."""
+    import ctypes
+
+    from paper_1004_0480_gb300 import _lib as L
+    from paper_1004_0480_gb300.sim import Batch, Sim
+    if tsteps == 2 and (stencil == 19 or model == "ch_front"):
+        pytest.skip("one step per launch")
+    out = (ctypes.c_int64 * 2)()
+    lib = L.load()
+    for ty in (6, 8, 12, 14):
+        # 2 x 512 work items at least: more than the GPU holds
+        sims = [Sim(W.with_(MAKE[model]((64, 8 * ty, 64), i), stencil=stencil), storage)
+                for i in range(2)]
+        b = Batch(model, storage)
+        b.set_tuning(tsteps=tsteps, tile_q=16, tile_y=ty, zchunk=1)
+        for s in sims:
+            b.add(s)
+        assert lib.rd_debug_batch_grid(b.b, out) == L.RD_EINVAL      # nothing launched yet
+        b.step(tsteps)
+        b.sync()
+        assert lib.rd_debug_batch_grid(b.b, out) == L.RD_OK
+        assert out[0] == min(1024, out[1]), (ty, list(out))
+        b.close()
+        for s in sims:
+            s.close()
