@@ -206,7 +206,7 @@ rd_status rd_create(const rd_config* cfg, rd_ctx** out);
  * planes of ny rows of ``pitch`` elements (float32 or bfloat16), pitch = nx
  * rounded up to a multiple of 128 bytes, x fastest.  Level 0 is current
  * after rd_set_field and after every even number of kernel launches.  Until
- * a tuning is set (rd_get_tuning then reports one step per launch) a context
+ * a tiling is set (rd_get_tuning then reports one step per launch) a context
  * on attached memory leaves the levels as one launch per step would: the
  * current one by the parity of the steps, the step before in the other. */
 rd_status rd_attach(rd_ctx* ctx, void* state, void* scratch);
@@ -294,10 +294,11 @@ rd_status rd_set_step_count(rd_ctx* ctx, int64_t n);
  * rd_set_tuning validates; RD_EINVAL if the CTA or its shared memory does
  * not fit one SM.  A new context starts with tsteps 1, tile_y 14 (12 for
  * the Cahn-Hilliard models), graph 1, regcap 0 and the z-chunk whose work
- * items fill the resident CTA slots in the fewest waves.  Until a tuning is
- * set (rd_set_tuning, rd_autotune) the library may step with another tiling
- * and with two steps per launch where its cost model expects that to be
- * faster: the results are the same bits, rd_launch_count is lower. */
+ * items fill the resident CTA slots in the fewest waves.  Until another
+ * tiling is set (rd_set_tuning with another tsteps, tile_q, tile_y or zchunk
+ * than rd_get_tuning reports; rd_autotune) the library may step with another
+ * tiling and with two steps per launch where its cost model expects that to
+ * be faster: the results are the same bits, rd_launch_count is lower. */
 typedef struct rd_tuning {
     int32_t tsteps, tile_q, tile_y, zchunk, graph;
     int32_t regcap;   /* 0 or 1; no effect: each kernel has its own register
