@@ -1461,6 +1461,9 @@ rd_status rd_autotune(rd_ctx* c, rd_tuning* best_out) {
             }
         }
       }
+    // what a context steps with untuned (two steps at most per launch): the
+    // tuning kept is then never slower than none
+    const rd_tuning plan = default_plan(g, default_tuning(g), 2);
     cudaEvent_t e0, e1;
     RD_CUDA(c, cudaEventCreate(&e0));
     RD_CUDA(c, cudaEventCreate(&e1));
@@ -1491,8 +1494,52 @@ rd_status rd_autotune(rd_ctx* c, rd_tuning* best_out) {
         std::sort(rates.begin(), rates.end());
         return rates[rates.size() / 2];
     };
-    // pass 1: every candidate, briefly; pass 2: the best few, median of
-    // several longer timings (one short timing is too noisy to rank tilings
+    // the same of a graph of ``reps`` launches, replayed, as rd_step runs
+    // them: single launches of a small grid measure the host
+    auto time_replayed = [&](const rd_tuning& t, int reps, int samples) -> double {
+        c->tun = t;
+        c->desc_dirty = true;
+        if (upload_desc(c) != RD_OK) return -1.0;
+        if (!c->capture_stream &&
+            cudaStreamCreateWithFlags(&c->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
+            cudaGetLastError();
+            return -1.0;
+        }
+        if (cudaStreamBeginCapture(c->capture_stream, cudaStreamCaptureModeThreadLocal) !=
+            cudaSuccess) {
+            cudaGetLastError();
+            return -1.0;
+        }
+        const int64_t before = c->launches;
+        rd_status st = RD_OK;
+        for (int i = 0; i < reps && st == RD_OK; ++i)
+            st = launch_ctx(c, t.tsteps, c->cur, c->capture_stream);
+        const int64_t launches = c->launches - before;
+        c->launches = before;                               // captured, not run
+        cudaGraph_t gr = nullptr;
+        cudaGraphExec_t exec = nullptr;
+        bool ok = cudaStreamEndCapture(c->capture_stream, &gr) == cudaSuccess && st == RD_OK &&
+                  cudaGraphInstantiate(&exec, gr, 0) == cudaSuccess;
+        std::vector<double> rates;
+        for (int k = -1; k < samples && ok; ++k) {          // the first one warms up
+            cudaEventRecord(e0, c->stream);
+            ok = cudaGraphLaunch(exec, c->stream) == cudaSuccess;
+            cudaEventRecord(e1, c->stream);
+            ok = ok && cudaEventSynchronize(e1) == cudaSuccess;
+            c->launches += launches;
+            float ms = 0;
+            if (ok) cudaEventElapsedTime(&ms, e0, e1);
+            if (k >= 0) rates.push_back(cells * t.tsteps * reps / (ms * 1e-3) / 1e9);
+        }
+        if (exec) cudaGraphExecDestroy(exec);
+        if (gr) cudaGraphDestroy(gr);
+        cudaGetLastError();
+        if (!ok) return -1.0;
+        std::sort(rates.begin(), rates.end());
+        return rates[rates.size() / 2];
+    };
+    // pass 1: every candidate, briefly; pass 2: the best few and the plan,
+    // median of several replays (one short timing is too noisy to rank tilings
     // a few percent apart)
     std::vector<std::pair<double, rd_tuning>> ranked;
     for (const rd_tuning& t : cands) {
@@ -1506,10 +1553,12 @@ rd_status rd_autotune(rd_ctx* c, rd_tuning* best_out) {
                      [](const auto& x, const auto& y) { return x.first > y.first; });
     double best = -1.0;
     rd_tuning bt = saved;
-    const size_t finalists = std::min<size_t>(ranked.size(), 8);
-    for (size_t i = 0; i < finalists; ++i) {
-        const rd_tuning& t = ranked[i].second;
-        const double rate = time_tuning(t, 8, 5);
+    if (ranked.size() > 8) ranked.resize(8);
+    ranked.push_back({0.0, plan});
+    for (const auto& r : ranked) {
+        const rd_tuning& t = r.second;
+        double rate = time_replayed(t, kGraphLaunches, 5);
+        if (rate < 0) rate = time_tuning(t, 8, 5);
         if (std::getenv("RD_AUTOTUNE_VERBOSE"))
             std::fprintf(stderr, "rd_autotune %s final T=%d tile_y=%d zchunk=%d regcap=%d: %.2f GLUPS\n",
                          key.c_str(), t.tsteps, t.tile_y, t.zchunk, t.regcap, rate);
