@@ -470,8 +470,8 @@ rd_status rd_batch_remove(rd_batch* b, rd_ctx* ctx);
 int32_t rd_batch_size(const rd_batch* b);
 /* Enqueue on ``stream`` (NULL = legacy default stream). */
 rd_status rd_batch_set_stream(rd_batch* b, void* stream);
-/* Tuning shared by all members (tile_q, tile_y, zchunk, tsteps, graph,
- * regcap).  Without it a batch uses one step per launch, the default tile
+/* Tuning shared by all members (tile_q, tile_y, zchunk, tsteps, graph).
+ * Without it a batch uses one step per launch, the default tile
  * height and the z-chunk that fills the CTA slots in the fewest waves over
  * its current members. */
 rd_status rd_batch_set_tuning(rd_batch* b, const rd_tuning* t);

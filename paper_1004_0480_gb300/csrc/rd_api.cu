@@ -202,18 +202,17 @@ int variant_code(const rd_config& g) {
 // ``batch``: of the form that batches launch, whose register budgets differ
 // (LayoutM::regs): a plain 14-row diffusion kernel fits 4 CTAs on an SM alone
 // and 3 in a batch, a two-species one 3 and 2.
-int occupancy(int model, int storage, int T, int ty, int regcap = 0, int plain = 0,
-              int stencil = 7, int tq = kTileQ, bool batch = false) {
+int occupancy(int model, int storage, int T, int ty, int plain, int stencil, int tq = kTileQ,
+              bool batch = false) {
     static std::mutex mu;
-    static std::map<std::tuple<int, int, int, int, int, int, int, int, bool>, int> cache;
+    static std::map<std::tuple<int, int, int, int, int, int, int, bool>, int> cache;
     std::lock_guard<std::mutex> g(mu);
-    auto key = std::make_tuple(model, storage, T, ty, regcap, plain, stencil, tq, batch);
+    auto key = std::make_tuple(model, storage, T, ty, plain, stencil, tq, batch);
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;
     int occ = 0;
     LaunchArgs dummy{};
     dummy.use_one = !batch;
-    dummy.regcap = regcap;
     // plain: a variant_code
     dummy.plain = plain == 1;
     dummy.wind3 = plain == 2;
@@ -574,7 +573,7 @@ rd_tuning default_tuning(const rd_config& g) {
     t.tile_q = kTileQ;
     t.tile_y = default_tile_y(g.model);
     t.graph = 1;
-    const int occ = occupancy(g.model, g.storage, t.tsteps, t.tile_y, 0, variant_code(g),
+    const int occ = occupancy(g.model, g.storage, t.tsteps, t.tile_y, variant_code(g),
                               stencil_of(g));
     const long long cols = (long long)tiles(g.nx, kTileW) * tiles(g.ny, t.tile_y);
     t.zchunk = wave_zchunk({{cols, g.nz}}, (long long)std::max(occ, 1) * num_sms());
@@ -633,7 +632,7 @@ rd_tuning default_plan(const rd_config& g, const rd_tuning& t1, int maxT) {
             t.tile_y = ty;
             t.zchunk = 1;
             if (T > 2 || check_tuning(g, t) != RD_OK) continue;
-            const int occ = occupancy(g.model, g.storage, T, ty, 0, variant_code(g), sten);
+            const int occ = occupancy(g.model, g.storage, T, ty, variant_code(g), sten);
             if (occ < 1) continue;
             const PlaneCost pc = plane_cost(g, T);
             // an SM's time per plane with ``ctas`` work items on it
@@ -842,7 +841,6 @@ rd_status launch_ctx(rd_ctx* c, int T, int parity, cudaStream_t st, Use use = Us
     a.use_one = 1;
     a.one = use == Use::kPlan ? c->plan_desc : use == Use::kPlan1 ? c->plan1_desc : c->desc;
     a.nitems = items_of(a.one);
-    a.regcap = t.regcap;
     a.plain = plain_problem(c->cfg);
     a.wind3 = c->cfg.wind_kind == RD_WIND_3D;
     a.windx = windx_problem(c->cfg);
@@ -870,8 +868,7 @@ rd_status launch_ctx(rd_ctx* c, int T, int parity, cudaStream_t st, Use use = Us
     const int sten = stencil_of(c->cfg);
     const size_t sm = smem_of(c->cfg.model, c->cfg.storage, T, a.ty, sten, t.tile_q);
     const int occ = std::max(
-        1, occupancy(c->cfg.model, c->cfg.storage, T, a.ty, a.regcap,
-                     variant_code(c->cfg), sten, t.tile_q));
+        1, occupancy(c->cfg.model, c->cfg.storage, T, a.ty, variant_code(c->cfg), sten, t.tile_q));
     const long long grid = std::min<long long>(a.nitems, (long long)occ * num_sms());
     cudaError_t e =
         launch_model(c->cfg.model, c->cfg.storage, T, a, (int)grid, sm, st, nullptr, sten);
@@ -881,8 +878,8 @@ rd_status launch_ctx(rd_ctx* c, int T, int parity, cudaStream_t st, Use use = Us
 }
 
 long long ctx_graph_key(const rd_ctx* c, const rd_tuning& t) {
-    return ((((((long long)t.tsteps * 64 + t.tile_q) * 64 + t.tile_y) * 100000 + t.zchunk) * 2 +
-             t.regcap) * 4 + c->kernel);
+    return ((((long long)t.tsteps * 64 + t.tile_q) * 64 + t.tile_y) * 100000 + t.zchunk) * 4 +
+           c->kernel;
 }
 
 constexpr int kGraphLaunches = 16;
@@ -1442,7 +1439,7 @@ rd_status rd_autotune(rd_ctx* c, rd_tuning* best_out) {
             rd_tuning t{};
             t.tsteps = T; t.tile_q = tq; t.tile_y = ty; t.graph = 1; t.zchunk = 1;
             if (check_tuning(g, t) != RD_OK) continue;
-            const int occ = occupancy(g.model, g.storage, T, ty, 0, variant_code(g), sten, tq);
+            const int occ = occupancy(g.model, g.storage, T, ty, variant_code(g), sten, tq);
             if (occ < 1) continue;
             // z-chunks for 1, 2, 4, 8 waves of CTAs; for the one- and two-step
             // kernels also every split of z into 1..16 chunks, since how
@@ -1545,8 +1542,8 @@ rd_status rd_autotune(rd_ctx* c, rd_tuning* best_out) {
     for (const rd_tuning& t : cands) {
         const double rate = time_tuning(t, 4, 1);
         if (std::getenv("RD_AUTOTUNE_VERBOSE"))
-            std::fprintf(stderr, "rd_autotune %s T=%d tile_y=%d zchunk=%d regcap=%d: %.2f GLUPS\n",
-                         key.c_str(), t.tsteps, t.tile_y, t.zchunk, t.regcap, rate);
+            std::fprintf(stderr, "rd_autotune %s T=%d tile_q=%d tile_y=%d zchunk=%d: %.2f GLUPS\n",
+                         key.c_str(), t.tsteps, t.tile_q, t.tile_y, t.zchunk, rate);
         if (rate > 0) ranked.push_back({rate, t});
     }
     std::stable_sort(ranked.begin(), ranked.end(),
@@ -1560,8 +1557,8 @@ rd_status rd_autotune(rd_ctx* c, rd_tuning* best_out) {
         double rate = time_replayed(t, kGraphLaunches, 5);
         if (rate < 0) rate = time_tuning(t, 8, 5);
         if (std::getenv("RD_AUTOTUNE_VERBOSE"))
-            std::fprintf(stderr, "rd_autotune %s final T=%d tile_y=%d zchunk=%d regcap=%d: %.2f GLUPS\n",
-                         key.c_str(), t.tsteps, t.tile_y, t.zchunk, t.regcap, rate);
+            std::fprintf(stderr, "rd_autotune %s final T=%d tile_q=%d tile_y=%d zchunk=%d: %.2f GLUPS\n",
+                         key.c_str(), t.tsteps, t.tile_q, t.tile_y, t.zchunk, rate);
         if (rate > best) { best = rate; bt = t; }
     }
     cudaEventDestroy(e0);
@@ -1738,7 +1735,7 @@ rd_tuning batch_tuning(rd_batch* b) {
     t.tile_q = kTileQ;
     t.tile_y = default_tile_y(b->model);
     t.graph = 1;
-    const int occ = occupancy(b->model, b->storage, 1, t.tile_y, 0, batch_variant(b), b->stencil,
+    const int occ = occupancy(b->model, b->storage, 1, t.tile_y, batch_variant(b), b->stencil,
                               kTileQ, true);
     std::vector<std::pair<long long, int>> cols_nz;
     for (rd_ctx* c : b->members)
@@ -1825,7 +1822,6 @@ rd_status batch_launch(rd_batch* b, const rd_tuning& t, int T, int parity, long 
     a.ninst = (int)b->members.size();
     a.parity = parity;
     a.nitems = nitems;
-    a.regcap = t.regcap;
     const int variant = batch_variant(b);
     a.plain = variant == 1;
     a.wind3 = variant == 2;
@@ -1833,7 +1829,7 @@ rd_status batch_launch(rd_batch* b, const rd_tuning& t, int T, int parity, long 
     a.vw = vw_of(t.tile_q);
     const size_t sm = smem_of(b->model, b->storage, T, a.ty, b->stencil, t.tile_q);
     const int occ = std::max(
-        1, occupancy(b->model, b->storage, T, a.ty, a.regcap, variant, b->stencil, t.tile_q, true));
+        1, occupancy(b->model, b->storage, T, a.ty, variant, b->stencil, t.tile_q, true));
     const long long grid = std::min<long long>(nitems, (long long)occ * num_sms());
     b->last = a;
     b->last_T = T;

@@ -68,7 +68,6 @@ struct LaunchArgs {
     long long nitems;          // total work items over all instances
     int ty;                    // tile height in rows (width is kTileQ vectors)
     int use_one;               // 1: a single instance, described by ``one``
-    int regcap;                // no effect (rd_tuning.regcap)
     int plain;                 // every instance has no held layer, source or
                                // wind, and isotropic diffusivities
     int wind3;                 // some instance has the 3-D wind (kernels take
