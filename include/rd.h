@@ -206,7 +206,7 @@ rd_status rd_create(const rd_config* cfg, rd_ctx** out);
  * planes of ny rows of ``pitch`` elements (float32 or bfloat16), pitch = nx
  * rounded up to a multiple of 128 bytes, x fastest.  Level 0 is current
  * after rd_set_field and after every even number of kernel launches.  Until
- * a tiling is set (rd_get_tuning then reports one step per launch) a context
+ * a tuning is set (rd_get_tuning then reports one step per launch) a context
  * on attached memory leaves the levels as one launch per step would: the
  * current one by the parity of the steps, the step before in the other. */
 rd_status rd_attach(rd_ctx* ctx, void* state, void* scratch);
@@ -294,11 +294,13 @@ rd_status rd_set_step_count(rd_ctx* ctx, int64_t n);
  * rd_set_tuning validates; RD_EINVAL if the CTA or its shared memory does
  * not fit one SM.  A new context starts with tsteps 1, tile_y 14 (12 for
  * the Cahn-Hilliard models), graph 1, regcap 0 and the z-chunk whose work
- * items fill the resident CTA slots in the fewest waves.  Until another
- * tiling is set (rd_set_tuning with another tsteps, tile_q, tile_y or zchunk
- * than rd_get_tuning reports; rd_autotune) the library may step with another
- * tiling and with two steps per launch where its cost model expects that to
- * be faster: the results are the same bits, rd_launch_count is lower. */
+ * items fill the resident CTA slots in the fewest waves.  Until a tuning is
+ * set (rd_set_tuning, rd_autotune) the library may step with another tiling
+ * and with two steps per launch where its cost model expects that to be
+ * faster: the results are the same bits, rd_launch_count is lower.  Setting
+ * the tuning that rd_get_tuning reports asks for that tuning itself;
+ * rd_set_graph changes the graph flag alone, in the library's own choice
+ * too. */
 typedef struct rd_tuning {
     int32_t tsteps, tile_q, tile_y, zchunk, graph;
     int32_t regcap;   /* 0 or 1; no effect: each kernel has its own register
@@ -306,6 +308,7 @@ typedef struct rd_tuning {
 } rd_tuning;
 rd_status rd_get_tuning(const rd_ctx* ctx, rd_tuning* out);
 rd_status rd_set_tuning(rd_ctx* ctx, const rd_tuning* t);
+rd_status rd_set_graph(rd_ctx* ctx, int32_t graph);
 
 /* Time a built-in list of tunings on this context's problem (launches read
  * the current level and write the spare level, so the state is unchanged)

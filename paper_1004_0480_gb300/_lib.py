@@ -92,6 +92,7 @@ SIGNATURES = {
     "rd_batch_step_each": (_I, [_P, ctypes.POINTER(ctypes.c_int64)]),
     "rd_batch_sync": (_I, [_P]),
     "rd_batch_destroy": (_I, [_P]),
+    "rd_set_graph": (_I, [_P, _I32]),
     "rd_batch_launch_count": (_I64, [_P]),
     "rd_debug_batch_grid": (_I, [_P, ctypes.POINTER(ctypes.c_int64)]),
     "rd_moments_noalloc": (_I, [_P, _I32, _I32, _I32, _I32, _I64, _P, _P]),

@@ -1391,17 +1391,16 @@ rd_status rd_set_tuning(rd_ctx* c, const rd_tuning* t) {
     if (!c || !t) return fail(c, RD_EINVAL, "null argument");
     rd_status st = check_tuning(c->cfg, *t);
     if (st != RD_OK) return fail(c, st, "%s", g_err);
-    const rd_tuning old = c->tun;
     c->tun = *t;
     c->tun.zchunk = std::min(c->tun.zchunk, c->cfg.nz);
-    // the same tiling with another graph flag, or what was read written back,
-    // asks for no tiling: the library's own plan stays
-    if (c->plan.tsteps && c->tun.tsteps == old.tsteps && c->tun.tile_q == old.tile_q &&
-        c->tun.tile_y == old.tile_y && c->tun.zchunk == old.zchunk)
-        c->plan.graph = c->plan1.graph = c->tun.graph;
-    else
-        c->plan.tsteps = 0;
+    c->plan.tsteps = 0;
     c->desc_dirty = true;
+    return RD_OK;
+}
+
+rd_status rd_set_graph(rd_ctx* c, int32_t graph) {
+    if (!c) return fail(nullptr, RD_EINVAL, "null context");
+    c->tun.graph = c->plan.graph = c->plan1.graph = graph;
     return RD_OK;
 }
 

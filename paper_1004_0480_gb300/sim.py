@@ -218,6 +218,11 @@ class Sim:
         return t.as_dict()
 
     def set_tuning(self, **kw):
+        """Set the named tuning fields; the graph flag alone leaves the tiling
+        (the library's own, unless one was set) as it is."""
+        if set(kw) == {"graph"}:
+            self._check(self.lib.rd_set_graph(self.ctx, kw["graph"]), "rd_set_graph")
+            return
         cur = self.tuning()
         cur.update(kw)
         t = L.RdTuning(cur["tsteps"], cur["tile_q"], cur["tile_y"], cur["zchunk"],
