@@ -613,8 +613,8 @@ constexpr double kLaunchUs = 1.9, kPlaneUs = 0.45;
 // What a context steps with while its tuning is the default one: the tile
 // height, z-chunk and steps per launch (at most ``maxT``) of the least
 // modelled cost per step.  Small grids take short chunks (a 97 x 65 x 50
-// Brusselator: 10 rows x 5 planes, 2.7 us a step, where 14 rows x 8 planes
-// at one step per launch took 9.8), large ones the fewest waves; two steps
+// zero-flux Brusselator: 2.6 us a step, where 14 rows x 8 planes at one step
+// per launch took 9.8), large ones the fewest waves; two steps
 // per launch halve the launches and the traffic, but three-species and
 // bfloat16 problems are bound by their arithmetic and keep one where the
 // launch gap does not decide.

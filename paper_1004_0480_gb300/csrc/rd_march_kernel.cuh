@@ -32,9 +32,9 @@
 //
 // Measured at 2 steps per launch against the one-step kernel before it
 // (4-cell vectors, one halo warp, scalar arithmetic), best tilings: 256^3
-// Brusselator FP32 376 -> 488 GLUPS, 512^3 diffusion 814 -> 1127, 192^3
-// Turing 294 -> 442, a 97 x 65 x 50 Brusselator 32 -> 107; at one step per
-// launch 376 -> 387 (HBM), BF16 428 -> 457.
+// Brusselator FP32 376 -> 504 GLUPS, 512^3 diffusion 814 -> 1124, 192^3
+// Turing 294 -> 454, a 97 x 65 x 50 zero-flux Brusselator 32 -> 120; at one
+// step per launch 376 -> 386 (HBM), BF16 428 -> 455.
 //
 // Boundary rules: rows and planes beyond a zero-flux y or z face are copied
 // in by mirror extension to distance T, so level 1 evaluated on a ghost
@@ -100,7 +100,8 @@ template <class M, class ST, int T> struct LayoutM {
     static constexpr int P = 5;           // planes issued ahead of plane e - 1
     // Registers a thread may take.  The march is bound by latency (16 warps
     // on an SM at 128 registers), so what lets another CTA in pays for a few
-    // spills.  Measured, GLUPS, at the best tiling of each:
+    // spills.  Measured when the budgets were chosen (the kernel has gained a
+    // few per cent since), GLUPS, at the best tiling of each:
     //   diffusion 512^3 FP32, T = 2: 933 (128) 935 (112) 986 (96) 1080 (80)
     //                         T = 1: 665 (96) 735 (80) 802 (64)
     //   Brusselator 256^3 FP32, T = 2: 433 (128) 427 (112) 478 (96) 401 (80)
@@ -303,9 +304,9 @@ struct PlaneFeed {
 // What a problem may have beside reactions and diffusion, so that the kernel
 // tests for nothing else: kPlain: no held layer, point source or wind, every
 // species isotropic; kWindX: no held layer, wind along +x or none, every
-// species anisotropic (the air problem, 512 x 512 x 64: 253 GLUPS, 0.90 of
-// the HBM copy rate, against 197 in the general variant); kWind3: the 3-D wind (upwind along y
-// and z too; T = 1); kGeneral: anything else.
+// species anisotropic (the air problem, 512 x 512 x 64: 249 GLUPS, 0.88 of
+// the HBM copy rate, against 197 in the general variant); kWind3: the 3-D wind
+// (upwind along y and z too; T = 1); kGeneral: anything else.
 enum MarchVar { kGeneral, kPlain, kWind3, kWindX };
 
 template <class M, class ST, int T, bool ONE, int VAR>

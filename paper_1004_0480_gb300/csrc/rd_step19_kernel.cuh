@@ -24,8 +24,8 @@
 //
 // Measured against the kernel before it (scalar arithmetic, single-element
 // shared loads with a 4-way bank conflict, sums of the field rows moved from
-// register to register), best tilings: 192^3 Turing 248 -> 316 GLUPS, the
-// 192^3 Cahn-Hilliard step 84 -> 112, the 144 x 144 x 384 plume 194 -> 247.
+// register to register), best tilings: 192^3 Turing 248 -> 321 GLUPS, the
+// 192^3 Cahn-Hilliard step 84 -> 120, the 144 x 144 x 384 plume 194 -> 268.
 // It is bound by latency: 12 to 18 warps on an SM wait on one another's
 // barrier and on shuffles and shared loads.
 //
@@ -59,7 +59,8 @@ template <class M, class ST, int PASS> struct Layout19 {
     static constexpr int ROWB = row19_bytes(NS, (int)sizeof(ST), MUF);
     static_assert(ROWB % 16 == 0 && (NS * SPB) % 16 == 0, "16-byte vectors");
     static_assert(PASS == 0 || M::CH, "passes 1 and 2 are for Cahn-Hilliard models");
-    // registers a thread may take (measured best tilings, GLUPS): the
+    // registers a thread may take (GLUPS at the best tilings when the budgets
+    // were chosen; the kernel has gained up to 8 % since): the
     // one-species plume 250 (80) 239 (96) 231 (128); two-species Turing 192^3
     // 275 (80) 311 (96) 319 (128); the Cahn-Hilliard step 72 (80) 102 (128)
     static constexpr int regs() {

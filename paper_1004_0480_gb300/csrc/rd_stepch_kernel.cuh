@@ -29,9 +29,9 @@ template <class ST> struct LayoutCH {
     static constexpr int RING = 6;        // planes e - 1 .. e + 4
     static constexpr int P = RING - 1;    // planes issued ahead of plane e - 2
     // registers a thread may take; front 192^3 FP32, GLUPS at the best
-    // tiling: 200 (128), 208 (112), 158 (96); the kernel before it (mirrored
-    // ghosts element by element, loads with a 4-way conflict): 188; eight
-    // uneven fronts batched 145 against 113
+    // tiling when the budget was chosen (210 now): 200 (128), 208 (112), 158
+    // (96); the kernel before it (mirrored ghosts element by element, loads
+    // with a 4-way conflict): 188; eight uneven fronts batched 145 against 113
     static constexpr int regs(bool lean) { return lean && sizeof(ST) == 4 ? 112 : 128; }
     __host__ __device__ static size_t state_bytes(int ty) {
         return (size_t)RING * RM::plane_bytes(ty + 4);
