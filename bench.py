@@ -37,6 +37,9 @@ from paper_1004_0480_gb300 import workloads as W  # noqa: E402
 METRIC = "GLUPS (cell updates per second / 1e9), brusselator 256^3 FP32"
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 PROFILE_FILE = os.path.join(ROOT, "profiles", "rd_step_brusselator_256.md")
+# the ncu summaries of the benchmark's kernel, by steps per launch
+PROFILE_FILES = {1: PROFILE_FILE,
+                 2: os.path.join(ROOT, "profiles", "rd_step2_brusselator_256.md")}
 WORKLOAD = "brusselator_256^3_periodic_10000_steps"
 KERNEL_SOURCES = ["paper_1004_0480_gb300/csrc/rd_step_kernel.cuh",
                   "paper_1004_0480_gb300/csrc/rd_march_kernel.cuh",
@@ -108,14 +111,13 @@ def kernel_sha():
 
 def profiled_traffic(tsteps, tile_q, tile_y):
     """(DRAM bytes per launch, tuning they were taken at) from the committed
-    ncu summary, if it was taken on the current kernel source at the same
-    steps per launch and tile; else (None, None).  The register cap does not
-    change what the kernel reads and writes; the z-chunk changes only how
-    many halo planes are re-read (mostly from L2), so the tuning is reported
-    beside the number instead of being required to match."""
+    ncu summary of that many steps per launch, if it was taken on the current
+    kernel source at the same tile; else (None, None).  The z-chunk changes
+    only how many halo planes are re-read (mostly from L2), so the tuning is
+    reported beside the number instead of being required to match."""
     try:
-        text = open(PROFILE_FILE).read()
-    except OSError:
+        text = open(PROFILE_FILES[tsteps]).read()
+    except (KeyError, OSError):
         return None, None
     fields = {}
     for line in text.splitlines():
@@ -490,11 +492,15 @@ def _timed_steps(torch, sim, steps, reps=2):
 
 
 def _entry(cells, steps, seconds, bytes_per_cell_step, tuning=None, **kw):
+    """One workload of the extras.  ``bytes_per_cell_step`` is what one step
+    per launch moves; a launch of T steps moves it once, which is what
+    roofline_frac counts, as the headline's roofline does."""
     peak, _ = measured_peak()
     glups = cells * steps / seconds / 1e9
+    T = tuning["tsteps"] if tuning else 1
     d = {"glups": glups, "cells": cells, "steps": steps,
-         "bytes_per_cell_step": bytes_per_cell_step,
-         "roofline_frac": glups * bytes_per_cell_step / peak}
+         "bytes_per_cell_step": bytes_per_cell_step, "steps_per_launch": T,
+         "roofline_frac": glups * bytes_per_cell_step / T / peak}
     if tuning is not None:
         d["tuning"] = tuning
     d.update(kw)
@@ -503,7 +509,7 @@ def _entry(cells, steps, seconds, bytes_per_cell_step, tuning=None, **kw):
 
 def run_extras(args, Sim, Batch, torch):
     """The other workloads: GLUPS and fraction of the measured HBM peak
-    (algorithmic bytes 2 x species x bytes per value per cell-step)."""
+    (algorithmic bytes 2 x species x bytes per value per cell and launch)."""
     out = {}
     # Brusselator 256^3 with BF16 storage (8 B per cell-step)
     cfg = W.cfg_brusselator_256()
