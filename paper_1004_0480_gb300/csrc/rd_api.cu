@@ -8,6 +8,7 @@
 
 #include <algorithm>
 #include <chrono>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -325,8 +326,8 @@ int periodic_axis(const rd_config& c, int s, int a) {
 
 // elements per row: rows padded to 128 bytes so 16-byte vectors never cross a
 // row end
-int pitch_of(const rd_config& g) {
-    return (int)align_up((size_t)g.nx, (size_t)(128 / elem_bytes(g.storage)));
+long long pitch_of(const rd_config& g) {
+    return (long long)align_up((size_t)g.nx, (size_t)(128 / elem_bytes(g.storage)));
 }
 
 rd_status validate(const rd_config* c) {
@@ -354,8 +355,9 @@ rd_status validate(const rd_config* c) {
     }
     if (c->storage != RD_STORE_F32 && c->storage != RD_STORE_BF16)
         return fail(nullptr, RD_EINVAL, "unknown storage %d", c->storage);
-    if (!plane_fits((long long)pitch_of(*c) * c->ny))
-        return fail(nullptr, RD_EINVAL, "grid too large: a plane of %d padded rows", c->ny);
+    if (pitch_of(*c) > INT_MAX || !plane_fits(pitch_of(*c) * c->ny))
+        return fail(nullptr, RD_EINVAL, "grid too large: %d rows of %lld elements a plane", c->ny,
+                    pitch_of(*c));
     for (int s = 0; s < c->nspecies; ++s) {
         for (int f = 0; f < 6; ++f)
             if (c->bc[s][f] < RD_BC_NEUMANN || c->bc[s][f] > RD_BC_DIRICHLET)
@@ -462,7 +464,7 @@ void layout(rd_ctx* c) {
     c->S = g.nspecies;
     c->vec = vec_of(g.storage);
     c->ebytes = elem_bytes(g.storage);
-    c->pitch = pitch_of(g);
+    c->pitch = (int)pitch_of(g);
     c->plane = (long long)c->pitch * g.ny;
     c->field_bytes = align_up((size_t)c->plane * g.nz * c->ebytes, 256);
     c->state_bytes = c->field_bytes * 2 * c->S;

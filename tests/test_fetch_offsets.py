@@ -102,5 +102,7 @@ def test_planes_past_the_offsets_are_refused():
         assert query((2, 2**28 - 9, 2), storage) == L.RD_OK       # 2^34 padded elements in BF16
         assert query((92683, 92683, 2), storage) == L.RD_EINVAL   # more than 2^34 cells
         assert query((2, 2**29, 2), storage) == L.RD_EINVAL
+        assert query((2**31 - 1, 2, 2), storage) == L.RD_EINVAL   # padded past an int
+        assert query((2**31 - 64, 2, 2), storage) == L.RD_OK
     assert query((2, 2**28, 2), "f32") == L.RD_OK
     assert query((2, 2**28, 2), "bf16") == L.RD_EINVAL
